@@ -107,7 +107,9 @@ typedef struct {
                                 FP32 change is located by a Wittrick-Williams counting search
                                 (bisection on the number of negative eigenvalues of K below
                                 the pole-free bound min_i beta_i sqrt(1 + (pi/(k h_i))^2)),
-                                certified in FP64 by count 0 at V[n-1] and odd at V[n]; items
+                                certified by count 0 at V[n-1] and odd at V[n], each count
+                                proven by the error bound that the FP32 count carries or
+                                else decided on the FP64 count; items
                                 outside the bound take the linear screen of 1. Default: 2 */
     int32_t count_block;     /* precision 2: threads per block of the counting kernel, 64, 128
                                 or 256 (two lanes per item, items of a block consecutive;
@@ -118,7 +120,9 @@ typedef struct {
                                 in kernels of their own (one thread per item: every 6th
                                 wavelength of a model and its last by bisection, then
                                 the others from a guess between those two indices)
-                                before the certificate's; 2 as 1, and the items the
+                                before the certificate's, which takes the
+                                points that the search's error bound leaves
+                                open; 2 as 1, and the items the
                                 search passes straight to the linear FP32 scan (no count
                                 change below the bound, a mode below V[0]) take that
                                 scan, its check and the mode-count search on a second,
@@ -278,7 +282,8 @@ int masw_last_count_phases(const masw_batch* batch, float* ms);
  * screen saw none) from the most recent two-precision scan, host or device
  * buffer of n_items; a diagnostic of how well the screen locates roots.
  * Under plan precision 2, bit 30 (MASW_SCREEN_COUNTED) is set on items whose
- * index the counting search located and the FP64 count certified. */
+ * index the counting search located and the counts at V[n-1] and V[n] certified
+ * (proven by the FP32 count's error bound, or decided on the FP64 count). */
 #define MASW_SCREEN_COUNTED (1 << 30)
 int masw_last_scan_screen(masw_batch* batch, int32_t* n32);
 

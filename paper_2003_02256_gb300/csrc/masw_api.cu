@@ -52,7 +52,6 @@ struct masw_batch {
     std::vector<double> lambda, kvec;
     std::vector<int32_t> order_sorted, order_natural;
     std::vector<int32_t> search_order;  // anchors of the split search, then the others
-    std::vector<int32_t> layer_order;   // items by model, models ordered by layer count
     int32_t n_anchor = 0;
     std::vector<int64_t> grad_off;
 
@@ -65,7 +64,6 @@ struct masw_batch {
     int32_t* d_order_sorted = nullptr;
     int32_t* d_order_natural = nullptr;
     int32_t* d_search_order = nullptr;
-    int32_t* d_layer_order = nullptr;
     int64_t* d_grad_off = nullptr;
     int32_t* d_counter = nullptr;
     double* d_ct = nullptr;
@@ -94,6 +92,8 @@ struct masw_batch {
     int side_prio = 0;
     cudaEvent_t side_fork = nullptr, side_join = nullptr;
     int32_t* d_nsearch = nullptr;
+    int32_t* d_one = nullptr;
+    int32_t* d_two = nullptr;
     int32_t* d_search2 = nullptr;
     int32_t* d_unres2 = nullptr;
     int32_t* d_fallback2 = nullptr;
@@ -132,7 +132,6 @@ struct masw_batch {
         b.item_model = d_item_model;
         b.order = ordered ? d_order_sorted : d_order_natural;
         b.search_order = d_search_order;
-        b.layer_order = d_layer_order;
         b.n_anchor = n_anchor;
         b.grad_off = d_grad_off;
         b.n_models = n_models;
@@ -338,12 +337,11 @@ static void free_batch(masw_batch* B) {
     if (B->side) cudaStreamDestroy(B->side);
     void* ptrs[] = {B->d_layers, B->d_loff,  B->d_woff,  B->d_nlim,   B->d_k,
                     B->d_item_model, B->d_order_sorted, B->d_order_natural, B->d_search_order,
-                    B->d_layer_order,
                     B->d_grad_off,
                     B->d_counter, B->d_ct, B->d_idx, B->d_status, B->d_croot, B->d_rows, B->d_bs,
                     B->d_dphi, B->d_ce, B->d_misfit, B->d_gb, B->d_gh, B->d_layers32, B->d_layers_df,
                     B->d_n32, B->d_cert, B->d_search, B->d_unres, B->d_fallback, B->d_counters,
-                    B->d_nsearch, B->d_search2, B->d_unres2, B->d_fallback2, B->d_upd, B->d_upd_err,
+                    B->d_nsearch, B->d_one, B->d_two, B->d_search2, B->d_unres2, B->d_fallback2, B->d_upd, B->d_upd_err,
                     B->d_chg_ct, B->d_chg_idx, B->d_chg_status, B->d_chg_delta,
                     B->d_chg_counters, B->d_lk_ct, B->d_lk_idx};
     for (void* p : ptrs)
@@ -399,18 +397,22 @@ static ScanPlan to_scan_plan(const masw_batch* B, const masw_plan& p) {
     return s;
 }
 
+static ScanSide scan_side(const masw_batch* B, bool overlap) {
+    return ScanSide{B->side,       B->side_prio, B->side_fork, B->side_join,   B->d_nsearch, B->d_one,
+                    B->d_two,      B->d_search2, B->d_unres2,  B->d_fallback2, overlap};
+}
+
 // Enqueue one full scan (all items) with the given plan on stream s.
 static cudaError_t enqueue_scan(masw_batch* B, const masw_plan& p, cudaStream_t s,
                                 bool phase_events = false) {
     if (p.precision >= 1) {
         ScanOut o{B->d_ct, B->d_idx, B->d_status, B->d_cert};
-        ScanSide side{B->side, B->side_prio, B->side_fork, B->side_join,
-                      B->d_nsearch, B->d_search2, B->d_unres2, B->d_fallback2};
+        const ScanSide side = scan_side(B, true);
         return launch_screen_scan(B->dev(p.ordered != 0), o, to_scan_plan(B, p), B->d_layers32,
                                   B->d_n32, B->d_search, B->d_unres, B->d_fallback, B->d_counters,
                                   p.precision == 2, 0, (int)B->n_items, s,
                                   phase_events ? B->phase_ev : nullptr,
-                                  p.precision == 2 && p.count_split == 2 ? &side : nullptr);
+                                  &side);
     }
     if (p.persistent) {
         cudaError_t e = cudaMemsetAsync(B->d_counter, 0, sizeof(int32_t), s);
@@ -596,17 +598,6 @@ int masw_model_batch_create(const masw_models_desc* md, const masw_grid* grid, v
     for (int32_t m : by_layers)
         for (int32_t j = B->woff[m]; j < B->woff[m + 1]; ++j)
             if (!anchor(m, j)) B->search_order.push_back(j);
-    // The certificate's order: model by model, the fewest layers first
-    // (measured a little faster there than the other way round, beside the
-    // second stream's chain). Left out when the models come in that order
-    // already.
-    if (!std::is_sorted(B->n_layers.begin(), B->n_layers.end())) {
-        B->layer_order.reserve(nw);
-        std::stable_sort(by_layers.begin(), by_layers.end(),
-                         [&](int32_t a, int32_t b) { return B->n_layers[a] < B->n_layers[b]; });
-        for (int32_t m : by_layers)
-            for (int32_t j = B->woff[m]; j < B->woff[m + 1]; ++j) B->layer_order.push_back(j);
-    }
     B->order_sorted = B->order_natural;
     std::stable_sort(B->order_sorted.begin(), B->order_sorted.end(),
                      [&](int32_t x, int32_t y) { return cost[x] > cost[y]; });
@@ -627,13 +618,13 @@ int masw_model_batch_create(const masw_models_desc* md, const masw_grid* grid, v
         dev_alloc(&B->d_k, nw) || dev_alloc(&B->d_item_model, nw) ||
         dev_alloc(&B->d_order_sorted, nw) || dev_alloc(&B->d_order_natural, nw) ||
         dev_alloc(&B->d_search_order, nw) ||
-        (!B->layer_order.empty() && dev_alloc(&B->d_layer_order, nw)) ||
         dev_alloc(&B->d_grad_off, nw + 1) || dev_alloc(&B->d_counter, 1) ||
         dev_alloc(&B->d_ct, nw) || dev_alloc(&B->d_idx, nw) || dev_alloc(&B->d_status, nw) ||
         dev_alloc(&B->d_layers32, rec32.size()) || dev_alloc(&B->d_layers_df, recdf.size()) ||
         dev_alloc(&B->d_n32, nw) || dev_alloc(&B->d_cert, nw) ||
         dev_alloc(&B->d_search, nw) || dev_alloc(&B->d_unres, nw) || dev_alloc(&B->d_fallback, nw) ||
         dev_alloc(&B->d_counters, 2 * SCAN_COUNTERS) || dev_alloc(&B->d_nsearch, nw) ||
+        dev_alloc(&B->d_one, nw) || dev_alloc(&B->d_two, nw) ||
         dev_alloc(&B->d_search2, nw) || dev_alloc(&B->d_unres2, nw) ||
         dev_alloc(&B->d_fallback2, nw)) {
         free_batch(B);
@@ -654,8 +645,6 @@ int masw_model_batch_create(const masw_models_desc* md, const masw_grid* grid, v
     if (e == cudaSuccess) e = up(B->d_order_sorted, B->order_sorted.data(), nw * 4);
     if (e == cudaSuccess) e = up(B->d_order_natural, B->order_natural.data(), nw * 4);
     if (e == cudaSuccess) e = up(B->d_search_order, B->search_order.data(), nw * 4);
-    if (e == cudaSuccess && B->d_layer_order)
-        e = up(B->d_layer_order, B->layer_order.data(), nw * 4);
     if (e == cudaSuccess) e = up(B->d_grad_off, B->grad_off.data(), (nw + 1) * 8);
     if (e == cudaSuccess) e = cudaEventCreate(&B->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&B->ev1);
@@ -939,6 +928,7 @@ int masw_dispersion_plain(masw_batch* B, double* ct, int32_t* ct_idx, int32_t* s
     ScanOut o{B->d_ct, B->d_idx, B->d_status, B->d_cert};
     DevBatch d = B->dev(false);
     ScanPlan sp = to_scan_plan(B, p);
+    const ScanSide side = scan_side(B, false);
     B->phases_valid = false;  // the per-model launches record no phase events
     B->count_phases_valid = false;
     B->side_phase_valid = false;
@@ -947,7 +937,7 @@ int masw_dispersion_plain(masw_batch* B, double* ct, int32_t* ct_idx, int32_t* s
         if (p.precision >= 1)
             CK(launch_screen_scan(d, o, sp, B->d_layers32, B->d_n32, B->d_search, B->d_unres,
                                   B->d_fallback, B->d_counters, p.precision == 2, B->woff[m],
-                                  B->woff[m + 1], B->stream, nullptr, nullptr));
+                                  B->woff[m + 1], B->stream, nullptr, &side));
         else
             CK(launch_scan(d, o, sp, B->d_counter, B->woff[m], B->woff[m + 1], B->stream));
         CK(cudaStreamSynchronize(B->stream));

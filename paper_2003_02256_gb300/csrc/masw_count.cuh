@@ -30,6 +30,7 @@
 //    serving tick scans linearly from `start`.
 #pragma once
 
+#include "masw_bound.cuh"
 #include "masw_device.cuh"
 #include "masw_df.cuh"
 #include "masw_screen.cuh"
@@ -97,14 +98,34 @@ __device__ __forceinline__ int count_search_pair(const float* __restrict__ lay32
     return pair_search(lay32, N, (float)k, (float)c0, (float)dc, -1, npf - 1, 1, half, pair);
 }
 
-// The search stage by one thread (the split search kernel): the same first
-// grid point in [0, npf) with a nonzero FP32 count, or -1, by bisection. One
-// point per step is one bit per evaluation, against log2(3)/2 for a pair's
-// three-way split, so an item takes about 20 % fewer evaluations; the pair
-// form stays where the certificate's lanes follow in the same kernel.
-__device__ __forceinline__ int count_search_single(const float* __restrict__ lay32, int N,
-                                                   double k, double c0, double dc, int npf) {
-    if (npf < 1) return -1;
+// What the split search knows of an item: its index n (the first grid point
+// in [0, npf) with a nonzero FP32 count, or -1) and which of the counts at
+// V[n-1] and V[n] the FP32 error bound proves (masw_bound.cuh).
+enum { PROOF_LO = 1, PROOF_HI = 2 };  // count 0 at V[n-1]; an odd count at V[n]
+struct Located {
+    int n;
+    int proof;  // PROOF_LO | PROOF_HI
+    int count;  // PROOF_HI: the count at V[n]
+};
+
+// FP32 count at grid point n with its error bound (the test velocity rounded
+// once from its FP64 value).
+__device__ __forceinline__ int count_bound_at(const float* __restrict__ lay32, int N, float kf,
+                                              double c0, double dc, int n, bool* sure) {
+    return inertia_bound_f(lay32, N, kf, (float)grid_c(c0, dc, n), sure);
+}
+
+// The search stage by one thread (the split search kernel): the first grid
+// point in [0, npf) with a nonzero FP32 count, or -1, by bisection. One point
+// per step is one bit per evaluation, against log2(3)/2 for a pair's three-way
+// split, so an item takes about 20 % fewer evaluations; the pair form stays
+// where the certificate's lanes follow in the same kernel. The bisection's
+// points take the plain count and the two points of the result the bounded
+// one: about 10 + 2 evaluations, the bounded one costing 1.5 plain ones.
+__device__ __forceinline__ Located count_search_single(const float* __restrict__ lay32, int N,
+                                                       double k, double c0, double dc, int npf) {
+    Located r{-1, 0, 0};
+    if (npf < 1) return r;
     const float kf = (float)k, c0f = (float)c0, dcf = (float)dc;
     // count 0 at lo (c = 0 when lo = -1), nonzero at hi; the top is taken as
     // nonzero and evaluated only when the bisection ends there (the change
@@ -115,8 +136,24 @@ __device__ __forceinline__ int count_search_single(const float* __restrict__ lay
         if (inertia_f(lay32, N, kf, fmaf((float)mid, dcf, c0f)) >= 1) hi = mid;
         else lo = mid;
     }
-    if (hi == npf - 1 && inertia_f(lay32, N, kf, fmaf((float)hi, dcf, c0f)) < 1) return -1;
-    return hi;
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        const int p = side ? lo : hi;
+        if (p < 0) break;
+        bool sure;
+        const int c = count_bound_at(lay32, N, kf, c0, dc, p, &sure);
+        if (side) {
+            if (sure && c == 0) r.proof |= PROOF_LO;
+        } else {
+            if (c < 1 && hi == npf - 1) return r;  // no change inside the range
+            if (sure && (c & 1)) {
+                r.proof |= PROOF_HI;
+                r.count = c;
+            }
+        }
+    }
+    r.n = hi;
+    return r;
 }
 
 // The guess for an item between two searched wavelengths of its model
@@ -134,51 +171,49 @@ __device__ __forceinline__ int search_guess(int na, int nb, int x, int d) {
 }
 
 // The search stage for an item between two searched wavelengths of its
-// model, from a guess g (search_guess; g < 0: a neighbour without an index,
-// and the item takes count_search_single). The count at g says on which
+// model, from a guess g (search_guess). The count at g says on which
 // side the change lies; steps of 1, 2, 4, ... from g away in that direction
 // bracket it, and bisection closes the bracket: 2 evaluations when g is the
 // change or the point below it, about 2 log2(e) + 2 for an error of e
 // points. The result is the same first nonzero point of a non-decreasing
-// count in [0, npf), or -1.
-__device__ __forceinline__ int count_search_guess(const float* __restrict__ lay32, int N,
-                                                  double k, double c0, double dc, int npf,
-                                                  int guess) {
-    if (npf < 1) return -1;
-    if (guess < 0) return count_search_single(lay32, N, k, c0, dc, npf);
-    const float kf = (float)k, c0f = (float)c0, dcf = (float)dc;
-    const int g = min(max(guess, 0), npf - 1);
-    int lo, hi;  // count 0 at lo (c = 0 when lo = -1), nonzero at hi
-    if (inertia_f(lay32, N, kf, fmaf((float)g, dcf, c0f)) >= 1) {
-        hi = g;
-        lo = -1;
-        for (int step = 1; hi > 0; step *= 2) {
-            const int p = max(hi - step, 0);
-            if (inertia_f(lay32, N, kf, fmaf((float)p, dcf, c0f)) < 1) {
-                lo = p;
-                break;
-            }
+// count in [0, npf), or -1. Every point takes the bounded count, so that the
+// two points of the result carry their proof with them (the plain count and
+// two bounded ones after it took 25 % longer). One place evaluates, so the
+// lanes of a warp stay together and the code compact.
+__device__ __forceinline__ Located count_search_guess(const float* __restrict__ lay32, int N,
+                                                      double k, double c0, double dc, int npf,
+                                                      int guess) {
+    Located r{-1, 0, 0};
+    if (npf < 1) return r;
+    const float kf = (float)k;
+    int lo = -1, hi = npf;  // count 0 at lo (c = 0 when lo = -1), nonzero at hi (not seen: npf)
+    int p = min(guess, npf - 1), step = 1;
+    bool down = false;
+    for (bool first = true;; first = false) {
+        bool sure;
+        const int c = count_bound_at(lay32, N, kf, c0, dc, p, &sure);
+        if (c >= 1) {
             hi = p;
-        }
-    } else {
-        lo = g;
-        hi = -1;
-        for (int step = 1; lo < npf - 1; step *= 2) {
-            const int p = min(lo + step, npf - 1);
-            if (inertia_f(lay32, N, kf, fmaf((float)p, dcf, c0f)) >= 1) {
-                hi = p;
-                break;
-            }
+            r.count = c;
+            r.proof = (r.proof & PROOF_LO) | ((sure && (c & 1)) ? PROOF_HI : 0);
+        } else {
             lo = p;
+            r.proof = (r.proof & PROOF_HI) | (sure ? PROOF_LO : 0);
         }
-        if (hi < 0) return -1;  // no change inside the range
+        if (first) down = c >= 1;
+        if (hi - lo <= 1) break;
+        if (down && lo < 0) {  // no lower end yet
+            p = max(hi - step, 0);
+            step *= 2;
+        } else if (!down && hi == npf) {  // no upper end yet
+            p = min(lo + step, npf - 1);
+            step *= 2;
+        } else {
+            p = lo + ((hi - lo) >> 1);
+        }
     }
-    while (hi - lo > 1) {
-        const int mid = lo + ((hi - lo) >> 1);
-        if (inertia_f(lay32, N, kf, fmaf((float)mid, dcf, c0f)) >= 1) hi = mid;
-        else lo = mid;
-    }
-    return hi;
+    if (hi < npf) r.n = hi;  // else no change inside the range
+    return r;
 }
 
 // The certificate stage for the search's index n (count_search_pair or

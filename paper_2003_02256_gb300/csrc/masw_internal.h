@@ -31,9 +31,6 @@ struct DevBatch {
     // then the others, bracketed by those neighbours
     const int32_t* search_order = nullptr;
     int32_t n_anchor = 0;
-    // all items, model by model from the fewest layers up (the split
-    // certificate's order over a whole batch), or nullptr
-    const int32_t* layer_order = nullptr;
 };
 
 // Items of a model between two fully searched ones in the split search.
@@ -80,23 +77,27 @@ struct ScanPlan {
 // that fail. n32, search, unresolved, fallback: n_items each; counters:
 // SCAN_COUNTERS per list set ([3]: fallback items, [5]: items that failed
 // their FP64 check).
-constexpr int SCAN_COUNTERS = 7;
+constexpr int SCAN_COUNTERS = 9;
 // n32 flag of an index located by the counting search (MASW_SCREEN_COUNTED)
 constexpr int32_t SCREEN_COUNTED = 1 << 30;
-// Plan count_split 2: a second stream for the items the counting search
-// passes straight to the linear FP32 scan. After the search kernel, `fork` on
-// the scan stream releases that stream; its fallback scan, check, mode-count
-// search and re-scan run (at priority `prio`, the stream's) beside the
-// certificate over lists of their own, and the scan stream waits for `join`
-// at the end. nsearch, search, unresolved, fallback: n_items each.
+// The split search's buffers (plan count_split 1 and 2: required; n_items
+// entries each) and, with overlap (count_split 2 over a whole batch), a second
+// stream for the items it passes straight to the linear FP32 scan. After the
+// search kernel, `fork` on the scan stream releases that stream; its fallback
+// scan, check, mode-count search and re-scan run (at priority `prio`, the
+// stream's) beside the certificate over lists of their own, and the scan
+// stream waits for `join` at the end.
 struct ScanSide {
     cudaStream_t s;
     int prio;
     cudaEvent_t fork, join;
     int32_t* nsearch;  // the search kernel's index per item (0: passed on)
+    int32_t* one;      // items with one of their two counts proven
+    int32_t* two;      // items with none
     int32_t* search;
     int32_t* unresolved;
     int32_t* fallback;
+    bool overlap;
 };
 // counters: 2 x SCAN_COUNTERS (the second set for the side stream's lists).
 cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPlan& p,
@@ -104,7 +105,7 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
                                int32_t* unresolved, int32_t* fallback, int32_t* counters,
                                int counting, int item_begin, int item_end, cudaStream_t s,
                                cudaEvent_t* phase_ev,  // nullptr or 3 events
-                               const ScanSide* side);  // nullptr: one stream
+                               const ScanSide* side);  // nullptr: fused plans only
 
 // Algorithm 1 continued: the first M sign changes per item with their
 // negative-eigenvalue count changes, from the first change `first` (the batch

@@ -518,6 +518,20 @@ __global__ void __launch_bounds__(256) fallback32_kernel(DevBatch b, const float
 }
 
 
+// Lists between the split search and its certificates (n_items entries each,
+// counts on the device).
+struct CountLists {
+    int32_t* n32;
+    int32_t* nsearch;  // the search's index per item (0: passed on)
+    int32_t* early;    // items for the linear FP32 scan
+    int32_t* n_early;
+    int32_t* one;      // items with one of the two counts proven (| ONE_LOW)
+    int32_t* n_one;
+    int32_t* two;      // items with none
+    int32_t* n_two;
+};
+constexpr int32_t ONE_LOW = 1 << 30;  // list `one`: V[n-1] is the point wanted
+
 // The counting search's FP64 certificate (plan precision 2), two lanes per
 // item (certify_pair; natural item order, or by layer count over a whole
 // batch: a warp's 16 items share a model and have adjacent wavelengths, so
@@ -539,8 +553,13 @@ __global__ void __launch_bounds__(256) fallback32_kernel(DevBatch b, const float
 // fewer spills), so that the block size also picks among the register
 // budgets.
 // Search stage alone (count_search_single or count_search_guess, one
-// thread per item): the index goes to nsearch[item], for
-// count_certify_kernel<B, true>. With an early list (plan count_split 2) the items the certificate would only pass on to
+// thread per item), with what its FP32 counts' error bound proves. An item
+// whose counts at V[n-1] (0) and V[n] (odd) are both proven is finished here.
+// With one of them proven it joins the list `one` (count_certify_one_kernel:
+// the other point in double-float), with none the list `two`
+// (count_certify_kernel). Bound by instruction issue (FP32, 88 % of cycles in
+// the first pass on the 8192-model ragged batch).
+// The items the certificate would only pass on to
 // the linear FP32 scan (no count change inside the pole-free range, a mode
 // below V[0], test routing 1..3) go straight to that list with their start in
 // n32, and nsearch gets 0 for them and for models without a scan range
@@ -550,13 +569,12 @@ __global__ void __launch_bounds__(256) fallback32_kernel(DevBatch b, const float
 // PASS 0: the items [item_begin, item_end) in natural order; 1: the anchor
 // items of b.search_order (every SEARCH_STRIDE-th wavelength of a model and
 // its last), each searched in full; 2: the other items, each searched
-// from a guess between its two anchors' indices (count_search_guess),
-// after pass 1.
+// from a guess between its two anchors' indices (count_search_guess; a
+// neighbour without an index: in full), after pass 1.
 template <int B, int PASS>
 __global__ void __launch_bounds__(B) count_search_kernel(DevBatch b,
                                                          const float* __restrict__ layers32,
-                                                         int32_t* nsearch, ScanOut o, int32_t* n32,
-                                                         int32_t* early, int32_t* n_early,
+                                                         ScanOut o, CountLists w,
                                                          int item_begin, int item_end) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     int item;
@@ -572,38 +590,81 @@ __global__ void __launch_bounds__(B) count_search_kernel(DevBatch b,
     const int N = b.model_loff[m + 1] - lo_rec - 1;
     const int nlim = b.model_nlim[m];
     if (nlim < 2) {
-        if (early) {
-            nsearch[item] = 0;
-            n32[item] = -1;
-            write_result(b, o, item, -1);
-            if (o.cert_counts) o.cert_counts[item] = -1;
-        }
+        w.nsearch[item] = 0;
+        w.n32[item] = -1;
+        write_result(b, o, item, -1);
+        if (o.cert_counts) o.cert_counts[item] = -1;
         return;
     }
     const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
     const double k = b.k[item];
     const int npf = pole_free_points_f(lay32, N, (float)k, (float)b.c0, (float)b.dc, nlim);
-    int n;
+    Located r;
     if (PASS == 2) {
         const int w0 = b.model_woff[m], w1 = b.model_woff[m + 1];
         const int ja = w0 + ((item - w0) / SEARCH_STRIDE) * SEARCH_STRIDE;
         const int jb = min(ja + SEARCH_STRIDE, w1 - 1);
-        const int na = nsearch[ja], nb = nsearch[jb];
+        const int na = w.nsearch[ja], nb = w.nsearch[jb];
+        // (a neighbour without an index: the middle of the range, then the
+        // doubling steps and bisection, any guess gives the same result)
         const int guess = (na >= 1 && nb >= 1) ? max(search_guess(na, nb, item - ja, jb - ja), 0)
-                                               : -1;
-        n = count_search_guess(lay32, N, k, b.c0, b.dc, npf, guess);
+                                               : npf >> 1;
+        r = count_search_guess(lay32, N, k, b.c0, b.dc, npf, guess);
     } else {
-        n = count_search_single(lay32, N, k, b.c0, b.dc, npf);
+        r = count_search_single(lay32, N, k, b.c0, b.dc, npf);
     }
-    if (!early || (n >= 1 && route_level(b.route) < 1)) {
-        nsearch[item] = n;
+    if (r.n < 1 || route_level(b.route) >= 1) {
+        // the start certify_pair gives these items (test routing: V[0])
+        w.nsearch[item] = 0;
+        w.n32[item] = (route_level(b.route) < 1 && npf >= 1 && r.n < 0) ? npf : 0;
+        if (o.cert_counts) o.cert_counts[item] = -1;
+        w.early[atomicAdd(w.n_early, 1)] = item;
         return;
     }
-    // the start certify_pair gives these items (test routing: V[0])
-    nsearch[item] = 0;
-    n32[item] = (route_level(b.route) < 1 && npf >= 1 && n < 0) ? npf : 0;
-    if (o.cert_counts) o.cert_counts[item] = -1;
-    early[atomicAdd(n_early, 1)] = item;
+    w.nsearch[item] = r.n;
+    if (r.proof == (PROOF_LO | PROOF_HI)) {
+        w.n32[item] = r.n | SCREEN_COUNTED;
+        write_result(b, o, item, r.n);
+        if (o.cert_counts) o.cert_counts[item] = pack_counts(0, r.count);
+    } else if (r.proof) {
+        // the count at V[n], when proven, rides in cert_counts' place
+        w.one[atomicAdd(w.n_one, 1)] = item | (r.proof == PROOF_HI ? ONE_LOW : 0);
+        if (o.cert_counts) o.cert_counts[item] = r.count;
+    } else {
+        w.two[atomicAdd(w.n_two, 1)] = item;
+    }
+}
+
+// The listed items of which the search's FP32 bound proved one of the two
+// counts: the other one in double-float (det_inertia_dd), one thread per item.
+// ONE_LOW marks those whose V[n-1] is wanted. An item whose count there is
+// not the certificate's goes to the list `two` (an FP32 index off by one, or
+// an even count). A quarter of the ragged batch's items, so half as many
+// double-float evaluations as lanes in the pair kernel.
+template <int B>
+__global__ void __launch_bounds__(B, (B == 256 ? 2 : 896 / B))
+    count_certify_one_kernel(DevBatch b, ScanOut o, CountLists w) {
+    const int total = *w.n_one;
+    const int stride = gridDim.x * B;
+    for (int t = blockIdx.x * B + threadIdx.x; t < total; t += stride) {
+        const int e = w.one[t];
+        const int item = e & ~ONE_LOW;
+        const bool low = e & ONE_LOW;
+        const int m = b.item_model[item];
+        const int lo_rec = b.model_loff[m];
+        const int N = b.model_loff[m + 1] - lo_rec - 1;
+        const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
+        const int n = w.nsearch[item];
+        const int v = det_inertia_dd(records_df(b, lo_rec), lay, N, b.k[item],
+                                     grid_c(b.c0, b.dc, low ? n - 1 : n));
+        if (low ? v == 0 : (v > 0 && (v & 1))) {
+            w.n32[item] = n | SCREEN_COUNTED;
+            write_result(b, o, item, n);
+            if (o.cert_counts) o.cert_counts[item] = pack_counts(0, low ? o.cert_counts[item] : v);
+        } else {
+            w.two[atomicAdd(w.n_two, 1)] = item;
+        }
+    }
 }
 
 // Algorithm 1's first change of one item as the first odd jump of the FP64
@@ -626,42 +687,18 @@ static __device__ __noinline__ int pair_mode_search(const float* laydf, const do
     return res;
 }
 
-template <int B, bool SPLIT>
-__global__ void __launch_bounds__(B, (B == 256 ? 2 : (B == 64 && SPLIT ? 10 : 896 / B)))
-    count_certify_kernel(DevBatch b, const float* __restrict__ layers32, ScanOut o,
-                         int32_t* n32, const int32_t* nsearch, int early, int32_t* search,
-                         int32_t* n_search, int32_t* fallback, int32_t* n_fallback,
-                         int32_t* unresolved, int32_t* n_unresolved, int item_begin,
-                         int item_end) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    int item = item_begin + (t >> 1);
-    if (item >= item_end) return;  // both lanes of a pair leave together
-    // a whole batch in the order by layer count (a warp's pairs, one model's
-    // or like models' items, walk the same number of layers)
-    if (SPLIT && b.layer_order && item_begin == 0 && item_end == b.n_items)
-        item = b.layer_order[item];
-    // (early list: the search kernel has passed the item on, or written it)
-    if (SPLIT && early && nsearch[item] < 1) return;
-    const int half = t & 1;
-    const unsigned pair = 3u << ((threadIdx.x & 31) & 30);
-    const int m = b.item_model[item];
-    const int lo_rec = b.model_loff[m];
-    const int N = b.model_loff[m + 1] - lo_rec - 1;
-    const int nlim = b.model_nlim[m];
-    if (nlim < 2) {
-        if (!half) {
-            n32[item] = -1;
-            write_result(b, o, item, -1);
-            if (o.cert_counts) o.cert_counts[item] = -1;
-        }
-        return;
-    }
+// One item's certificate and its recovery by a pair of lanes, the search's
+// index ns given: the result, the fallback list, or the re-scan list.
+__device__ __forceinline__ void certify_item(const DevBatch& b, const float* __restrict__ layers32,
+                                             const ScanOut& o, int item, int m, int lo_rec, int N,
+                                             int nlim, int npf, int ns, int half, unsigned pair,
+                                             int32_t* n32, int32_t* search, int32_t* n_search,
+                                             int32_t* fallback, int32_t* n_fallback,
+                                             int32_t* unresolved, int32_t* n_unresolved) {
     const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
-    const float* laydf = b.layers_df ? b.layers_df + (size_t)lo_rec * LAYER_STRIDE_DF : nullptr;
+    const float* laydf = records_df(b, lo_rec);
     const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
     const double k = b.k[item];
-    const int npf = pole_free_points_f(lay32, N, (float)k, (float)b.c0, (float)b.dc, nlim);
-    const int ns = SPLIT ? nsearch[item] : count_search_pair(lay32, N, k, b.c0, b.dc, npf, half, pair);
     const PairCount r = certify_pair(lay32, laydf, lay, N, k, b.c0, b.dc, nlim, npf, ns, half, pair);
     // the certificate's own failures (the FP64 counts around the located
     // point fail, or two modes inside one interval with no odd count found
@@ -697,6 +734,44 @@ __global__ void __launch_bounds__(B, (B == 256 ? 2 : (B == 64 && SPLIT ? 10 : 89
     } else {
         n32[item] = r.start;
         fallback[atomicAdd(n_fallback, 1)] = item;
+    }
+}
+
+// SPLIT: the items of the list w.two (a device-side count, grid-stride);
+// otherwise the items [item_begin, item_end), with the search in the same
+// kernel.
+template <int B, bool SPLIT>
+__global__ void __launch_bounds__(B, (B == 256 ? 2 : (B == 64 && SPLIT ? 10 : 896 / B)))
+    count_certify_kernel(DevBatch b, const float* __restrict__ layers32, ScanOut o, CountLists w,
+                         int32_t* n32, int32_t* search, int32_t* n_search, int32_t* fallback,
+                         int32_t* n_fallback, int32_t* unresolved, int32_t* n_unresolved,
+                         int item_begin, int item_end) {
+    const int half = threadIdx.x & 1;
+    const unsigned pair = 3u << ((threadIdx.x & 31) & 30);
+    const int end = SPLIT ? *w.n_two : item_end - item_begin;
+    const int stride = SPLIT ? (gridDim.x * B) >> 1 : 0;
+    for (int t = (blockIdx.x * B + threadIdx.x) >> 1; t < end; t += stride) {
+        const int item = SPLIT ? w.two[t] : item_begin + t;  // both lanes of a pair together
+        const int m = b.item_model[item];
+        const int lo_rec = b.model_loff[m];
+        const int N = b.model_loff[m + 1] - lo_rec - 1;
+        const int nlim = b.model_nlim[m];
+        if (!SPLIT && nlim < 2) {
+            if (!half) {
+                n32[item] = -1;
+                write_result(b, o, item, -1);
+                if (o.cert_counts) o.cert_counts[item] = -1;
+            }
+            return;
+        }
+        const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
+        const double k = b.k[item];
+        const int npf = pole_free_points_f(lay32, N, (float)k, (float)b.c0, (float)b.dc, nlim);
+        const int ns =
+            SPLIT ? w.nsearch[item] : count_search_pair(lay32, N, k, b.c0, b.dc, npf, half, pair);
+        certify_item(b, layers32, o, item, m, lo_rec, N, nlim, npf, ns, half, pair, n32, search,
+                     n_search, fallback, n_fallback, unresolved, n_unresolved);
+        if (!SPLIT) return;
     }
 }
 
@@ -846,36 +921,44 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
                                cudaEvent_t* phase_ev, const ScanSide* side) {
     if (item_end <= item_begin) return cudaSuccess;
     // counters: [0] screen queue, [1] unresolved count, [2] resolve queue,
-    // [3] fallback count, [4] fallback queue, [5] search count, [6] search queue;
-    // then the same for the side stream's lists
+    // [3] fallback count, [4] fallback queue, [5] search count, [6] search queue,
+    // [7] items with one count proven, [8] with none; then [0..6] for the side
+    // stream's lists
     cudaError_t e = cudaMemsetAsync(counters, 0, 2 * SCAN_COUNTERS * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
     int wpb = p.warps_per_block;
     int blocks = p.persistent ? p.blocks : (item_end - item_begin + wpb - 1) / wpb;
     size_t shm = (size_t)wpb * p.stage_layers * LAYER_STRIDE32 * sizeof(float);
     int n = item_end - item_begin;
-    const bool overlap = counting && p.count_split == 2 && side != nullptr;
+    const bool overlap = counting && p.count_split == 2 && side != nullptr && side->overlap;
     if (counting) {
+        if (p.count_split && !side) return cudaErrorInvalidValue;
         const int cb = p.count_block;
         const int grid = (2 * n + cb - 1) / cb;
         int32_t* const side_counters = counters + SCAN_COUNTERS;
-        int32_t* const nsearch = overlap ? side->nsearch : n32;
+        CountLists w{};
+        w.n32 = n32;
         if (p.count_split) {
-            int32_t* const el = overlap ? side->fallback : nullptr;
-            int32_t* const nel = overlap ? side_counters + 3 : nullptr;
+            w.nsearch = side->nsearch;
+            w.early = overlap ? side->fallback : fallback;
+            w.n_early = (overlap ? side_counters : counters) + 3;
+            w.one = side->one;
+            w.n_one = counters + 7;
+            w.two = side->two;
+            w.n_two = counters + 8;
             if (b.search_order && item_begin == 0 && item_end == b.n_items) {
                 // anchors first, then the items between them
                 const int na = b.n_anchor, nr = b.n_items - b.n_anchor;
                 if (na > 0)
                     count_search_kernel<128, 1><<<(na + 127) / 128, 128, 0, s>>>(
-                        b, layers32, nsearch, o, n32, el, nel, item_begin, item_end);
+                        b, layers32, o, w, item_begin, item_end);
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
                 if (nr > 0)
                     count_search_kernel<128, 2><<<(nr + 127) / 128, 128, 0, s>>>(
-                        b, layers32, nsearch, o, n32, el, nel, item_begin, item_end);
+                        b, layers32, o, w, item_begin, item_end);
             } else {
                 count_search_kernel<128, 0><<<(n + 127) / 128, 128, 0, s>>>(
-                    b, layers32, nsearch, o, n32, el, nel, item_begin, item_end);
+                    b, layers32, o, w, item_begin, item_end);
             }
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if (phase_ev && (e = cudaEventRecord(phase_ev[2], s)) != cudaSuccess) return e;
@@ -889,10 +972,17 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
             if (e != cudaSuccess) return e;
             if ((e = cudaEventRecord(side->join, side->s)) != cudaSuccess) return e;
         }
+        // the listed items, a few per thread: as many blocks as stay resident
+        const int sms = p.sms > 0 ? p.sms : 152;
+        const int per_sm = cb == 256 ? 2 : cb == 128 ? 7 : 10;
+        const int lgrid = std::max(1, std::min(grid, per_sm * sms));
 #define MASW_COUNT_LAUNCH(BS, SPL)                                                              \
-    count_certify_kernel<BS, SPL><<<grid, BS, 0, s>>>(b, layers32, o, n32, nsearch, overlap ? 1 : 0, \
-                                                      search, counters + 5, fallback, counters + 3, \
-                                                      unresolved, counters + 1, item_begin, item_end)
+    do {                                                                                        \
+        if (SPL) count_certify_one_kernel<BS><<<lgrid, BS, 0, s>>>(b, o, w);                    \
+        count_certify_kernel<BS, SPL><<<SPL ? lgrid : grid, BS, 0, s>>>(                        \
+            b, layers32, o, w, n32, search, counters + 5, fallback, counters + 3, unresolved,   \
+            counters + 1, item_begin, item_end);                                                \
+    } while (0)
         switch (cb * 2 + (p.count_split ? 1 : 0)) {
             case 128: MASW_COUNT_LAUNCH(64, false); break;
             case 129: MASW_COUNT_LAUNCH(64, true); break;
