@@ -77,7 +77,7 @@ struct ScanPlan {
 // that fail. n32, search, unresolved, fallback: n_items each; counters:
 // SCAN_COUNTERS per list set ([3]: fallback items, [5]: items that failed
 // their FP64 check).
-constexpr int SCAN_COUNTERS = 9;
+constexpr int SCAN_COUNTERS = 11;
 // n32 flag of an index located by the counting search (MASW_SCREEN_COUNTED)
 constexpr int32_t SCREEN_COUNTED = 1 << 30;
 // The split search's buffers (plan count_split 1 and 2: required; n_items

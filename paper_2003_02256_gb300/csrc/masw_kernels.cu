@@ -25,9 +25,12 @@
 //                         FP32 scan) and verify64_list_kernel (the check), for
 //                         large batches on a second stream beside the
 //                         certificate.
-//  first_count64_kernel   both two-precision plans: items that failed a check,
-//                         search on the mode count from V[0] (FP32-located,
-//                         FP64-certified rises).
+//  sign_scan_kernel       both two-precision plans: items that failed a check,
+//                         Algorithm 1 over FP32 signs with an error bound,
+//                         the points it leaves open in FP64.
+//  first_count64_kernel   the items with too many such points: search on the
+//                         mode count from V[0] (FP32-located, FP64-certified
+//                         rises).
 //  resolve64_kernel       items whose FP64 counts failed: FP64 scan from V[0].
 // Beyond the first change:
 //  changes_count64_kernel higher modes, FP32 search on the mode count, each
@@ -190,7 +193,8 @@ cudaError_t launch_scan(const DevBatch& b, const ScanOut& o, const ScanPlan& p, 
 // its fallback items take fallback32_kernel (linear FP32 scan) and
 // verify64_list_kernel (the check of 2. over the list); uncertified and
 // unverified items go to the search list.
-// Both: first_count64_kernel searches the listed items' first change on the
+// Both: sign_scan_kernel walks the listed items' grid on proven signs and
+// hands a few on to first_count64_kernel, which searches the first change on the
 // mode count from V[0] (each rise located on the FP32 count, certified on the
 // FP64 count); items whose FP64 counts fail take
 // resolve64_kernel, the FP64 scan from V[0].
@@ -540,9 +544,7 @@ constexpr int32_t ONE_LOW = 1 << 30;  // list `one`: V[n-1] is the point wanted
 // change lies above the pole-free range or at V[0] go to the fallback list
 // (linear FP32 scan and mode-count check); the certificate's own failures
 // (the counts around the located point, or an even count with no odd one
-// found above it) take the mode-count search from V[0] in this kernel
-// (pair_mode_search), and those whose FP64 counts fail there the FP64
-// re-scan list. Certified items keep SCREEN_COUNTED in n32. B threads per
+// found above it) to the sign scan's list. Certified items keep SCREEN_COUNTED in n32. B threads per
 // block (plan count_block: 64, 128 or 256), each block's B/2 items
 // consecutive, so its warps share the records of one or two models in L1;
 // the launch bounds ask for 896 resident threads per SM (at most 73
@@ -672,8 +674,7 @@ __global__ void __launch_bounds__(B, (B == 256 ? 2 : 896 / B))
 // V[top], then next_change_f32 (masw_modes.cuh), each rise of T located on
 // its FP32 value and certified on the FP64 count. *bad: the FP64 counts
 // failed (rescaling, or T not monotone at the evaluated points). Out of line:
-// first_count64_kernel runs it for listed items, the certificate for its own
-// few failures.
+// first_count64_kernel runs it for its listed items.
 static __device__ __noinline__ int pair_mode_search(const float* laydf, const double* lay,
                                                     const float* lay32, int N, double k,
                                                     double c0, double dc, int top, int half,
@@ -687,39 +688,18 @@ static __device__ __noinline__ int pair_mode_search(const float* laydf, const do
     return res;
 }
 
-// One item's certificate and its recovery by a pair of lanes, the search's
-// index ns given: the result, the fallback list, or the re-scan list.
+// One item's certificate by a pair of lanes, the search's index ns given: the
+// result, the search list (sign_scan_kernel), or the fallback list.
 __device__ __forceinline__ void certify_item(const DevBatch& b, const float* __restrict__ layers32,
                                              const ScanOut& o, int item, int m, int lo_rec, int N,
                                              int nlim, int npf, int ns, int half, unsigned pair,
                                              int32_t* n32, int32_t* search, int32_t* n_search,
-                                             int32_t* fallback, int32_t* n_fallback,
-                                             int32_t* unresolved, int32_t* n_unresolved) {
+                                             int32_t* fallback, int32_t* n_fallback) {
     const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
     const float* laydf = records_df(b, lo_rec);
     const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
     const double k = b.k[item];
     const PairCount r = certify_pair(lay32, laydf, lay, N, k, b.c0, b.dc, nlim, npf, ns, half, pair);
-    // the certificate's own failures (the FP64 counts around the located
-    // point fail, or two modes inside one interval with no odd count found
-    // above them): the mode-count search from V[0] right here, by this pair,
-    // while the kernel's other blocks run, where the fallback chain after the
-    // kernel would take three more launches in a row
-    if (route_level(b.route) < 1 && r.cert < 1 && (r.n >= 1 || (r.start >= 1 && r.start < npf))) {
-        bool bad;
-        const int res = pair_mode_search(laydf, lay, lay32, N, k, b.c0, b.dc, nlim - 1, half, pair,
-                                         &bad);
-        if (half) return;
-        if (o.cert_counts) o.cert_counts[item] = -1;
-        if (bad) {  // the FP64 scan from V[0]
-            n32[item] = 0;
-            unresolved[atomicAdd(n_unresolved, 1)] = item;
-        } else {
-            n32[item] = res;
-            write_result(b, o, item, res);
-        }
-        return;
-    }
     if (half) return;
     if (o.cert_counts) o.cert_counts[item] = route_level(b.route) >= 1 ? -1 : r.counts;
     if (route_level(b.route) >= 1) {  // test routing: every item through the linear FP32 scan from V[0]
@@ -728,7 +708,9 @@ __device__ __forceinline__ void certify_item(const DevBatch& b, const float* __r
     } else if (r.cert >= 1) {
         n32[item] = r.cert | SCREEN_COUNTED;
         write_result(b, o, item, r.cert);
-    } else if (r.n >= 1) {
+    } else if (r.n >= 1 || (r.start >= 1 && r.start < npf)) {
+        // the counts around the located point fail, or two modes inside one
+        // interval with no odd count found above them
         n32[item] = r.n;
         search[atomicAdd(n_search, 1)] = item;
     } else {
@@ -744,8 +726,7 @@ template <int B, bool SPLIT>
 __global__ void __launch_bounds__(B, (B == 256 ? 2 : (B == 64 && SPLIT ? 10 : 896 / B)))
     count_certify_kernel(DevBatch b, const float* __restrict__ layers32, ScanOut o, CountLists w,
                          int32_t* n32, int32_t* search, int32_t* n_search, int32_t* fallback,
-                         int32_t* n_fallback, int32_t* unresolved, int32_t* n_unresolved,
-                         int item_begin, int item_end) {
+                         int32_t* n_fallback, int item_begin, int item_end) {
     const int half = threadIdx.x & 1;
     const unsigned pair = 3u << ((threadIdx.x & 31) & 30);
     const int end = SPLIT ? *w.n_two : item_end - item_begin;
@@ -770,15 +751,13 @@ __global__ void __launch_bounds__(B, (B == 256 ? 2 : (B == 64 && SPLIT ? 10 : 89
         const int ns =
             SPLIT ? w.nsearch[item] : count_search_pair(lay32, N, k, b.c0, b.dc, npf, half, pair);
         certify_item(b, layers32, o, item, m, lo_rec, N, nlim, npf, ns, half, pair, n32, search,
-                     n_search, fallback, n_fallback, unresolved, n_unresolved);
+                     n_search, fallback, n_fallback);
         if (!SPLIT) return;
     }
 }
 
-// Items that failed their FP64 check (the counting search's certificate or
-// the three-point mode-count check of a linear FP32 scan; mostly items with
-// an even jump of the mode count below their first change, a mode trapped in
-// a low-velocity layer next to a pole of that layer): Algorithm 1's first
+// Items that the sign scan hands on (too many points its error bound leaves
+// open): Algorithm 1's first
 // change as the first odd jump of the FP64 mode count T = s + 2 J0 above V[0].
 // A pair of lanes per item (pairs pop the list): the FP64 counts at V[0] and
 // V[top], then next_change_f32 (masw_modes.cuh), which locates each rise of T
@@ -823,6 +802,126 @@ __global__ void __launch_bounds__(32) first_count64_kernel(DevBatch b, ScanOut o
                 write_result(b, o, item, res);
             }
         }
+    }
+}
+
+// Algorithm 1 over proven signs, for the items that failed a check: mostly
+// items with modes trapped in a low-velocity layer, each a root of det K and a
+// pole of that layer inside one grid interval, so an even jump of the mode
+// count without a sign change. One block per item, one grid point per thread
+// and round: the FP32 count with its error bound gives the sign (the count's
+// parity) wherever the bound proves it, and the few points it leaves open
+// below the first change take the FP64 count of det_inertia_df, the block's
+// threads one point each. The first point whose sign differs from V[0]'s is
+// the change. Inside the pole-free range [0, npf) the count never decreases:
+// equal counts at its two ends leave no change between, and the walk starts at
+// its end. An item that needs more than SIGN_SCAN_BUDGET FP64 counts (thin
+// layers at long wavelengths, few events) goes on to the mode-count search
+// (first_count64_kernel), one whose FP64 count fails to the FP64 re-scan.
+// The search visits every event of the mode count in turn, a pair of lanes
+// per item: on 32,000 items of models with inverted speeds (1,000 extreme
+// models, 9,546 listed items) it took 50 ms, here 1.5 ms; 0.80 and 0.11 ms on
+// the 121 listed items of a 701-model ragged batch, 1.16 and 0.16 ms on the
+// 1,463 of the 8192-model one. Bound by FP32 instruction issue, on short
+// lists by the latency of a round (about 25 us at 30 layers).
+constexpr int SIGN_SCAN_THREADS = 128;
+constexpr int SIGN_SCAN_BUDGET = 1024;
+__global__ void __launch_bounds__(SIGN_SCAN_THREADS, 4)
+    sign_scan_kernel(DevBatch b, ScanOut o, const float* __restrict__ layers32, int32_t* n32,
+                     const int32_t* __restrict__ list, const int32_t* __restrict__ n_list,
+                     int32_t* counter, int32_t* hard, int32_t* n_hard, int32_t* unresolved,
+                     int32_t* n_unresolved) {
+    __shared__ float s_lay[32 * LAYER_STRIDE32];  // records of up to 31 layers
+    __shared__ int s_item, s_first, s_open, s_bad, s_end[2];
+    __shared__ int s_list[SIGN_SCAN_THREADS];
+    const int tid = threadIdx.x;
+    const int total = *n_list;
+    if (total == 0) return;  // uniform across the block
+    for (;;) {
+        if (tid == 0) {
+            s_item = atomicAdd(counter, 1);
+            s_bad = 0;
+        }
+        __syncthreads();
+        const int t = s_item;
+        if (t >= total) return;
+        const int item = list[t];
+        if (route_level(b.route) >= 2) {  // test routing: every item to the mode-count search
+            if (tid == 0) hard[atomicAdd(n_hard, 1)] = item;
+            __syncthreads();
+            continue;
+        }
+        const int m = b.item_model[item];
+        const int lo_rec = b.model_loff[m];
+        const int N = b.model_loff[m + 1] - lo_rec - 1;
+        const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
+        const float* laydf = records_df(b, lo_rec);
+        const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
+        if (N < 32) {
+            for (int q = tid; q < (N + 1) * LAYER_STRIDE32; q += SIGN_SCAN_THREADS) s_lay[q] = lay32[q];
+            lay32 = s_lay;
+        }
+        __syncthreads();
+        const double k = b.k[item];
+        const float kf = (float)k;
+        const int nlim = b.model_nlim[m];  // >= 2 for listed items
+        const int npf = pole_free_points_f(lay32, N, kf, (float)b.c0, (float)b.dc, nlim);
+        // the counts at V[0] and at the end of the pole-free range, a warp each
+        if (tid < 64) {
+            const int p = tid < 32 ? 0 : max(npf - 1, 0);
+            bool sure;
+            int c = count_bound_at(lay32, N, kf, b.c0, b.dc, p, &sure);
+            if (!sure) c = det_inertia_df(laydf, lay, N, k, grid_c(b.c0, b.dc, p));
+            if ((tid & 31) == 0) s_end[tid >> 5] = c;
+        }
+        __syncthreads();
+        const int c0 = s_end[0];
+        const int carry = c0 & 1;
+        int base = (npf > 0 && s_end[1] == c0) ? npf : 1;
+        int res = -1, used = 0;
+        bool bad = c0 < 0, over = false;
+        for (; !bad && base < nlim; base += SIGN_SCAN_THREADS) {
+            if (tid == 0) {
+                s_first = 0x7fffffff;
+                s_open = 0;
+            }
+            __syncthreads();
+            const int n = base + tid;
+            bool sure = true;
+            int c = carry;
+            if (n < nlim) c = count_bound_at(lay32, N, kf, b.c0, b.dc, n, &sure);
+            const unsigned diff = __ballot_sync(FULL, sure && (c & 1) != carry);
+            if (diff && (tid & 31) == 0) atomicMin(&s_first, n + __ffs(diff) - 1);
+            if (!sure) s_list[atomicAdd(&s_open, 1)] = n;
+            __syncthreads();
+            const int first = s_first, open = s_open;
+            used += open;
+            over = used > SIGN_SCAN_BUDGET;
+            if (!over && tid < open && s_list[tid] < first) {
+                const int v = det_inertia_df(laydf, lay, N, k, grid_c(b.c0, b.dc, s_list[tid]));
+                if (v < 0) s_bad = 1;
+                else if ((v & 1) != carry) atomicMin(&s_first, s_list[tid]);
+            }
+            __syncthreads();
+            res = s_first;
+            bad = s_bad != 0;
+            __syncthreads();
+            if (over || bad || res != 0x7fffffff) break;
+            res = -1;
+        }
+        if (tid == 0) {
+            if (bad) {
+                n32[item] = 0;
+                unresolved[atomicAdd(n_unresolved, 1)] = item;
+            } else if (over) {
+                hard[atomicAdd(n_hard, 1)] = item;
+            } else {
+                n32[item] = res;
+                write_result(b, o, item, res);
+                if (o.cert_counts) o.cert_counts[item] = -1;
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -883,7 +982,8 @@ static cudaError_t launch_prio(void (*kernel)(Arg...), int grid, int block, size
 
 // The kernels after the screen or the counting kernels, over one set of
 // lists: (counting) the linear FP32 scan of the fallback list and its FP64
-// check, then the mode-count search of the items that failed a check and the
+// check, then the sign scan of the items that failed a check, the mode-count
+// search of those it hands on and the
 // FP64 re-scan of the items whose counts failed. phase_ev1: recorded after
 // the search (or nullptr).
 static cudaError_t launch_tail(const DevBatch& b, const ScanOut& o, const ScanPlan& p,
@@ -905,9 +1005,16 @@ static cudaError_t launch_tail(const DevBatch& b, const ScanOut& o, const ScanPl
     // (0.1 % and none of the ragged batch's items): one warp per block and up
     // to 8 blocks per SM spread the list over every SM, where blocks of
     // several warps would stack a list of a thousand items on a few SMs.
-    const int lblocks = std::max(1, std::min(8 * (p.sms > 0 ? p.sms : 152), n));
-    e = launch_prio(first_count64_kernel, lblocks, 32, 0, s, prio, b, o, n32, layers32, search,
-                    counters + 5, counters + 6, unresolved, counters + 1);
+    const int sms = p.sms > 0 ? p.sms : 152;
+    const int lblocks = std::max(1, std::min(8 * sms, n));
+    // (the fallback list is done with: it takes the items handed on)
+    int32_t* const hard = fallback;
+    e = launch_prio(sign_scan_kernel, std::max(1, std::min(4 * sms, n)), SIGN_SCAN_THREADS, 0, s,
+                    prio, b, o, layers32, n32, search, counters + 5, counters + 6, hard,
+                    counters + 9, unresolved, counters + 1);
+    if (e != cudaSuccess) return e;
+    e = launch_prio(first_count64_kernel, lblocks, 32, 0, s, prio, b, o, n32, layers32, hard,
+                    counters + 9, counters + 10, unresolved, counters + 1);
     if (e != cudaSuccess) return e;
     if (phase_ev1 && (e = cudaEventRecord(phase_ev1, s)) != cudaSuccess) return e;
     return launch_prio(resolve64_kernel, lblocks, 32, 0, s, prio, b, o, unresolved, counters + 1,
@@ -922,8 +1029,9 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
     if (item_end <= item_begin) return cudaSuccess;
     // counters: [0] screen queue, [1] unresolved count, [2] resolve queue,
     // [3] fallback count, [4] fallback queue, [5] search count, [6] search queue,
-    // [7] items with one count proven, [8] with none; then [0..6] for the side
-    // stream's lists
+    // [7] items with one count proven, [8] with none, [9] items the sign scan
+    // hands to the mode-count search, [10] their queue; then the same for the
+    // side stream's lists
     cudaError_t e = cudaMemsetAsync(counters, 0, 2 * SCAN_COUNTERS * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
     int wpb = p.warps_per_block;
@@ -980,8 +1088,8 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
     do {                                                                                        \
         if (SPL) count_certify_one_kernel<BS><<<lgrid, BS, 0, s>>>(b, o, w);                    \
         count_certify_kernel<BS, SPL><<<SPL ? lgrid : grid, BS, 0, s>>>(                        \
-            b, layers32, o, w, n32, search, counters + 5, fallback, counters + 3, unresolved,   \
-            counters + 1, item_begin, item_end);                                                \
+            b, layers32, o, w, n32, search, counters + 5, fallback, counters + 3, item_begin,   \
+            item_end);                                                                          \
     } while (0)
         switch (cb * 2 + (p.count_split ? 1 : 0)) {
             case 128: MASW_COUNT_LAUNCH(64, false); break;
