@@ -1067,17 +1067,17 @@ static int run_roots(masw_batch* B) {
     int rc;
     if ((rc = ensure(&B->d_croot, B->n_items))) return rc;
     if ((rc = run_scan(B))) return rc;
-    CK(launch_refine(B->dev(false), B->d_idx, 1e-13, B->d_croot, B->stream));
+    CK(launch_refine(B->dev(false), B->d_layers32, B->d_idx, 1e-13, B->d_croot, B->stream));
     return MASW_OK;
 }
 
 static int run_root_grad(masw_batch* B) {
     int rc;
     if ((rc = ensure(&B->d_rows, B->grad_len)) ||
-        (rc = ensure(&B->d_bs, 12 * (B->grad_len + B->n_items))))
+        (rc = ensure(&B->d_bs, root_grad_scratch((int)B->n_items, B->max_layers, B->sm_count))))
         return rc;
     if ((rc = run_roots(B))) return rc;
-    CK(launch_root_grad(B->dev(false), B->d_croot, B->d_rows, B->d_bs, B->stream));
+    CK(launch_root_grad(B->dev(false), B->d_croot, B->d_rows, B->d_bs, B->sm_count, B->stream));
     return MASW_OK;
 }
 

@@ -165,7 +165,9 @@ static __device__ __noinline__ ElemBound elem_bound_trig(float kh, float pp, flo
 struct BoundState { float p00, p01, p11, e; };
 
 // Eliminates one layer's top node: the number of negative eigenvalues of its
-// pivot; *sure is cleared when the pivot's inertia is not proven.
+// pivot; *sure is cleared when the pivot's inertia is not proven. BOUND false:
+// the recurrence alone.
+template <bool BOUND>
 __device__ __forceinline__ int bound_layer(BoundState& st, const float* __restrict__ L, float k,
                                            float c2, bool* sure) {
     const float4 LA = *reinterpret_cast<const float4*>(L);
@@ -225,6 +227,7 @@ __device__ __forceinline__ int bound_layer(BoundState& st, const float* __restri
     st.p00 = fmaf(2.0f, aE, st.p00) - fmaf(w00, t00, w10 * t10);
     st.p01 = st.p01 - fmaf(w00, t01, w10 * t11);
     st.p11 = fmaf(2.0f, dG, st.p11) - fmaf(w01, t01, w11 * t11);
+    if (!BOUND) return neg_eigs_2x2(det, s00);
     // the bound
     const float M = norm_2x2(n00, n01, n11);
     const float dO = o.ca * fmaf(fabsf(fm), o.tB, afr * o.tF);
@@ -250,14 +253,16 @@ __device__ __forceinline__ int bound_layer(BoundState& st, const float* __restri
 }
 
 // Negative eigenvalues of K(k, c) (inertia_f) with the running bound: *sure
-// is true when the count is proven. Requires c < beta_halfspace.
+// is true when the count is proven (BOUND false: not touched). Requires
+// c < beta_halfspace.
+template <bool BOUND = true>
 __device__ __forceinline__ int inertia_bound_f(const float* __restrict__ lay, int N, float k,
                                                float c, bool* sure) {
     const float c2 = c * c;
     BoundState st{0.0f, 0.0f, 0.0f, 0.0f};
     bool ok = true;
     int cnt = 0;
-    for (int j = 0; j < N; ++j) cnt += bound_layer(st, lay + j * LAYER_STRIDE32, k, c2, &ok);
+    for (int j = 0; j < N; ++j) cnt += bound_layer<BOUND>(st, lay + j * LAYER_STRIDE32, k, c2, &ok);
     const float4 LA = *reinterpret_cast<const float4*>(lay + N * LAYER_STRIDE32);
     const float q = c2 * lay[N * LAYER_STRIDE32 + 4], p = c2 * LA.w;
     const float s2 = 1.0f - q, r = sqrtf(1.0f - p), s = sqrtf(s2);
@@ -268,6 +273,7 @@ __device__ __forceinline__ int inertia_bound_f(const float* __restrict__ lay, in
     const float h01 = LA.y * iden * fmaf(g, q, -2.0f * den);
     const float s00 = st.p00 + h00, s01 = st.p01 + h01, s11 = st.p11 + h11;
     const float det = fmaf(s00, s11, -s01 * s01);
+    if (!BOUND) return cnt + neg_eigs_2x2(det, s00);
     const float mS = norm_2x2(s00, s01, s11);
     // the half-space block: its terms, and s = sqrt(1 - q), whose error is that of q over s
     const float mH = fmaxf(h00, h11) + LA.y * iden * fmaf(g, q, 2.0f * den) + rc2g * rsqrtf(s2);

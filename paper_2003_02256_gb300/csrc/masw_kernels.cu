@@ -1611,16 +1611,61 @@ __device__ __forceinline__ double det_rel(const double* __restrict__ lay, int N,
     return ldexp(f, d);
 }
 
+// A root's bracket narrowed on the FP32 count (inertia_bound_f's recurrence,
+// no bound): [a, bq] inside [lo, hi] with the count's parity changing across
+// it, a few FP32 steps wide, split in three per step by the pair's lanes. The
+// caller checks the FP64 determinant's signs at its ends. Returns false when
+// the FP32 parities at lo and hi agree.
+static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ lay32, int N,
+                                                     float kf, float lo, float hi, int half,
+                                                     unsigned pair, float* a_out, float* b_out) {
+    float a = lo, bq = hi;
+    int own = inertia_bound_f<false>(lay32, N, kf, half ? bq : a, nullptr) & 1;
+    const int oth = __shfl_xor_sync(pair, own, 1);
+    if (own == oth) return false;
+    const int par_a = half ? oth : own;
+    // down to two FP32 steps of the velocity (2^-22 relative): the count's own
+    // error is below that (about 1e-8 relative, from its misses next to roots)
+    while (bq - a > 2.4e-7f * bq) {
+        const float w = (bq - a) * (1.0f / 3.0f);
+        const float p0 = a + w, p1 = bq - w;
+        if (!(p0 > a && p1 < bq)) break;
+        own = inertia_bound_f<false>(lay32, N, kf, half ? p1 : p0, nullptr) & 1;
+        const int o = __shfl_xor_sync(pair, own, 1);
+        const int c0 = half ? o : own, c1 = half ? own : o;
+        if (c0 != par_a) {
+            bq = p0;
+        } else if (c1 != par_a) {
+            a = p0;
+            bq = p1;
+        } else {
+            a = p1;
+        }
+    }
+    *a_out = a;
+    *b_out = bq;
+    return true;
+}
+
 // Refined root inside [V[idx-1], V[idx]] (the change located by the scan) to
-// a bracket narrower than rel_tol * c, two lanes per item. Illinois (modified
+// a bracket narrower than rel_tol * c, two lanes per item. The bracket is
+// first narrowed on the FP32 count (bracket_root_f32, about 7 FP32 steps) and
+// widened by its error, and kept when the FP64 determinant changes sign
+// across it (else the scan's bracket). Then Illinois (modified
 // regula falsi) on det K, which has a simple zero there: the secant point x of
 // the bracket ends is evaluated a quarter tolerance on either side (one point
 // per lane); when the two straddle the zero the bracket closes, otherwise the
 // nearer point replaces the end of its sign, and an end kept twice in a row
 // has its value halved, so both ends converge. Every 8th step uses the
 // midpoint, so the bracket also shrinks at least as fast as in bisection.
-// Returns the midpoint of the final bracket; an exact zero returns its point.
-__global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const int32_t* __restrict__ idx,
+// Returns that secant point, or the midpoint of a bracket within the
+// tolerance; an exact zero returns its point.
+// Bound by the FP64 pipe: from the scan's bracket, closed by points a quarter
+// tolerance apart, it took about 7 pairs of
+// FP64 determinants (2.48 ms for 512 models of 12 layers and 150
+// wavelengths), from the FP32 bracket 2 (1.14 ms).
+__global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __restrict__ layers32,
+                                                     const int32_t* __restrict__ idx,
                                                      double rel_tol, double* croot) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int it = t >> 1;
@@ -1638,13 +1683,41 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const int32_t* 
     const int N = b.model_loff[m + 1] - lo_rec - 1;
     const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
     const double k = b.k[it];
-    double lo = grid_c(b.c0, b.dc, id - 1), hi = grid_c(b.c0, b.dc, id);
-    int e_own;
-    const double f_own = det_scaled(lay, N, k, half ? hi : lo, &e_own);
-    const double f_oth = __shfl_xor_sync(pair, f_own, 1);
-    const int e_oth = __shfl_xor_sync(pair, e_own, 1);
-    double f_lo = half ? f_oth : f_own, f_hi = half ? f_own : f_oth;
-    const int e_lo = half ? e_oth : e_own, e_hi = half ? e_own : e_oth;
+    const double v_lo = grid_c(b.c0, b.dc, id - 1), v_hi = grid_c(b.c0, b.dc, id);
+    double lo = v_lo, hi = v_hi;
+    bool narrow = false;
+    if (layers32) {
+        float a, c;
+        narrow = bracket_root_f32(layers32 + (size_t)lo_rec * LAYER_STRIDE32, N, (float)k,
+                                  (float)v_lo, (float)v_hi, half, pair, &a, &c);
+        if (narrow) {
+            const double pad = 1.8e-7 * v_hi;
+            lo = fmax(v_lo, (double)a - pad);
+            hi = fmin(v_hi, (double)c + pad);
+            narrow = lo < hi;
+        }
+        if (!narrow) {
+            lo = v_lo;
+            hi = v_hi;
+        }
+    }
+    double f_lo, f_hi;
+    int e_lo, e_hi;
+    for (;;) {
+        int e_own;
+        const double f_own = det_scaled(lay, N, k, half ? hi : lo, &e_own);
+        const double f_oth = __shfl_xor_sync(pair, f_own, 1);
+        const int e_oth = __shfl_xor_sync(pair, e_own, 1);
+        f_lo = half ? f_oth : f_own;
+        f_hi = half ? f_own : f_oth;
+        e_lo = half ? e_oth : e_own;
+        e_hi = half ? e_own : e_oth;
+        // the FP32 bracket stands when the FP64 signs at its ends differ
+        if (!narrow || (f_lo < 0.0 && f_hi > 0.0) || (f_lo > 0.0 && f_hi < 0.0)) break;
+        lo = v_lo;
+        hi = v_hi;
+        narrow = false;
+    }
     double result;
     if (!(f_lo == f_lo) || !(f_hi == f_hi) ||
         ((f_lo > 0.0) == (f_hi > 0.0) && f_lo != 0.0 && f_hi != 0.0)) {
@@ -1658,22 +1731,34 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const int32_t* 
         f_lo = ldexp(f_lo, e_lo - e_ref);
         f_hi = ldexp(f_hi, e_hi - e_ref);
         int side = 0;
+        result = nan;
         for (int i = 0; i < 200 && (hi - lo) > rel_tol * hi; ++i) {
             double x = (i % 8 == 7) ? 0.5 * (lo + hi) : hi - f_hi * (hi - lo) / (f_hi - f_lo);
             if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
-            const double eps = 0.25 * rel_tol * hi;
+            const double w = hi - lo, slope = (f_hi - f_lo) / w;
+            const double eps = fmax(0.25 * rel_tol * hi, 1e-3 * w);
             const double p0 = fmax(x - eps, lo + 0.25 * (x - lo));
             const double p1 = fmin(x + eps, hi - 0.25 * (hi - x));
             const double fp = det_rel(lay, N, k, half ? p1 : p0, e_ref);
             const double fq = __shfl_xor_sync(pair, fp, 1);
             const double f0 = half ? fq : fp, f1 = half ? fp : fq;
-            if (f0 == 0.0 || !(f0 == f0)) { lo = hi = p0; break; }
-            if (f1 == 0.0 || !(f1 == f1)) { lo = hi = p1; break; }
+            if (f0 == 0.0 || !(f0 == f0)) { result = p0; break; }
+            if (f1 == 0.0 || !(f1 == f1)) { result = p1; break; }
             if ((f0 > 0.0) != (f1 > 0.0)) {  // the zero lies between the two points
                 lo = p0;
                 hi = p1;
                 f_lo = f0;
                 f_hi = f1;
+                // The secant of the new bracket, v wide, is off by at most
+                // about C v^2 / 4, C = f''/(2 f') ~ |slope ratio - 1| / w:
+                // taken when that is below a tenth of the tolerance (with
+                // side 0 both slopes are the determinant's).
+                const double v = hi - lo, s1 = (f1 - f0) / v;
+                if (side == 0 && fabs(s1 - slope) * v * v < 0.4 * rel_tol * hi * w * fabs(s1)) {
+                    result = hi - f1 / s1;
+                    break;
+                }
+                side = 0;
             } else if ((f0 > 0.0) == (f_hi > 0.0)) {  // both on the upper end's side
                 hi = p0;
                 f_hi = f0;
@@ -1686,65 +1771,19 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const int32_t* 
                 side = -1;
             }
         }
-        result = 0.5 * (lo + hi);
+        if (!(result == result)) result = 0.5 * (lo + hi);
     }
     if (!half) croot[it] = result;
 }
 
-cudaError_t launch_refine(const DevBatch& b, const int32_t* idx, double rel_tol, double* croot,
-                          cudaStream_t s) {
+cudaError_t launch_refine(const DevBatch& b, const float* layers32, const int32_t* idx,
+                          double rel_tol, double* croot, cudaStream_t s) {
     if (b.n_items <= 0) return cudaSuccess;
-    refine_kernel<<<(2 * b.n_items + 127) / 128, 128, 0, s>>>(b, idx, rel_tol, croot);
+    refine_kernel<<<(2 * b.n_items + 127) / 128, 128, 0, s>>>(b, layers32, idx, rel_tol, croot);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------- root grad
-
-// 2x2 helpers for the (cold) adjoint path: general matrices m = {a, b, c, d}
-// = [[a, b], [c, d]].
-struct M2 { double a, b, c, d; };
-__device__ __forceinline__ M2 mmul(M2 x, M2 y) {
-    return {x.a * y.a + x.b * y.c, x.a * y.b + x.b * y.d, x.c * y.a + x.d * y.c, x.c * y.b + x.d * y.d};
-}
-__device__ __forceinline__ M2 madd(M2 x, M2 y) { return {x.a + y.a, x.b + y.b, x.c + y.c, x.d + y.d}; }
-__device__ __forceinline__ M2 msub(M2 x, M2 y) { return {x.a - y.a, x.b - y.b, x.c - y.c, x.d - y.d}; }
-__device__ __forceinline__ double mdet(M2 x) { return x.a * x.d - x.b * x.c; }
-// x^-1 y
-__device__ __forceinline__ M2 msolve(M2 x, M2 y) {
-    double id = 1.0 / mdet(x);
-    M2 adj = {x.d * id, -x.b * id, -x.c * id, x.a * id};
-    return mmul(adj, y);
-}
-__device__ __forceinline__ void mvsolve(M2 x, double v0, double v1, double* o0, double* o1) {
-    double id = 1.0 / mdet(x);
-    *o0 = (x.d * v0 - x.b * v1) * id;
-    *o1 = (-x.c * v0 + x.a * v1) * id;
-}
-__device__ __forceinline__ void ld(const double* p, M2* m) { *m = {p[0], p[1], p[2], p[3]}; }
-__device__ __forceinline__ void st(double* p, M2 m) { p[0] = m.a; p[1] = m.b; p[2] = m.c; p[3] = m.d; }
-
-// Element blocks of layer j at (k, c), k dropped: K11, K12 (K22 and K21 follow
-// from the layer's symmetry: K22 = [[A, -B], [-B, Dd]], K21 = K12^T).
-__device__ __forceinline__ void elem_blocks(const double* L, double k, double c2, M2* K11, M2* K12,
-                                            M2* K21, M2* K22) {
-    LayerNum n = layer_numerators(L, k, c2, inv_c2(c2));
-    double id = 1.0 / n.Dh;
-    double A = n.n00 * id, B = n.n01 * id, Dd = n.n11 * id;
-    double E = n.ce * id, F = n.cf * id, G = n.cg * id;
-    *K11 = {A, B, B, Dd};
-    *K22 = {A, -B, -B, Dd};
-    *K12 = {E, F, -F, G};
-    *K21 = {E, -F, F, G};
-}
-
-// The blocks of elem_blocks from its six stored entries (A, B, Dd, E, F, G).
-__device__ __forceinline__ void stored_blocks(const double* E6, M2* K11, M2* K12, M2* K21, M2* K22) {
-    const double A = E6[0], B = E6[1], Dd = E6[2], E = E6[3], F = E6[4], G = E6[5];
-    *K11 = {A, B, B, Dd};
-    *K22 = {A, -B, -B, Dd};
-    *K12 = {E, F, -F, G};
-    *K21 = {E, -F, F, G};
-}
 
 // One thread per item. Row layout: dC/dbeta_0..beta_N, dC/dh_0..h_{N-1}.
 // The null vector u of K(C*) comes from a twisted block factorization: a
@@ -1753,126 +1792,171 @@ __device__ __forceinline__ void stored_blocks(const double* E6, M2* K11, M2* K12
 // condensed block G_j = P_j + B_j is singular at the root, and the node
 // where it is most singular (relative to its size) carries the largest
 // amplitude. u starts there and is propagated upward with the top-down
-// factors and downward with the bottom-up ones, so it only ever decays and
+// factors T_j = S_j^-1 K12_j and downward with the bottom-up ones
+// Q_j = M_j^-1 K21_j, so it only ever decays and
 // neither a thick top layer (mode confined to the surface) nor a deep one
-// breaks it. Each layer's element entries are evaluated once (first sweep)
-// and kept for the other three sweeps. `bs` holds 24 doubles per node of the
-// item, starting at 12 * grad_off[item] + 12 * item = 24 * (sum of (N+1) of
-// earlier items).
-__global__ void __launch_bounds__(64) root_grad_kernel(DevBatch b, const double* __restrict__ croot,
-                                                       double* rows, double* bs) {
-    int it = blockIdx.x * blockDim.x + threadIdx.x;
-    if (it >= b.n_items) return;
-    int m = b.item_model[it];
-    int lo_rec = b.model_loff[m];
-    int N = b.model_loff[m + 1] - lo_rec - 1;
-    double* row = rows + b.grad_off[it];
-    double* ws = bs + 12 * b.grad_off[it] + 12 * (int64_t)it;
+// breaks it. Each layer's part of the implicit-function rule (elem_quad_grad)
+// is taken as u passes it. Bound by the FP64 pipe: about 300 FP64
+// instructions a layer, where the element's entries in dual numbers with
+// three directions, four sweeps over general 2x2 blocks and a division per
+// solve took about 850 (1.82 -> 0.86 ms for 512 models of 12 layers and 150
+// wavelengths).
+// Scratch: ROOT_SLOTS doubles per node and thread, node-major and a thread's
+// next to its neighbours', so that a warp's accesses are whole lines; the grid
+// strides over the items, so that the scratch stays within the L2.
+// Slots of node j: [0..3] T_j; [4..6] P_j; [7..12] layer j's entries, then
+// [7..10] Q_j; [0], [1] d q / d beta_j, d q / d h_j once T_j or Q_j is used.
+constexpr int ROOT_THREADS = 64;
+constexpr int ROOT_SLOTS = 13;
+__global__ void __launch_bounds__(ROOT_THREADS) root_grad_kernel(DevBatch b,
+                                                                 const double* __restrict__ croot,
+                                                                 double* rows, double* scratch) {
+    const int tid = blockIdx.x * ROOT_THREADS + threadIdx.x;
+    const int nt = gridDim.x * ROOT_THREADS;
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
-    double c = croot[it];
-    if (!(c == c)) {
-        for (int p = 0; p < 2 * N + 1; ++p) row[p] = nan;
-        return;
+    auto ws = [&](int node, int slot) -> double& {
+        return scratch[((size_t)node * ROOT_SLOTS + slot) * nt + tid];
+    };
+    for (int it = tid; it < b.n_items; it += nt) {
+        const int m = b.item_model[it];
+        const int lo_rec = b.model_loff[m];
+        const int N = b.model_loff[m + 1] - lo_rec - 1;
+        double* row = rows + b.grad_off[it];
+        const double c = croot[it];
+        if (!(c == c)) {
+            for (int p = 0; p < 2 * N + 1; ++p) row[p] = nan;
+            continue;
+        }
+        const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
+        const double k = b.k[it];
+        const double c2 = c * c;
+        const double ic2 = inv_c2(c2);
+        // top-down: P_j, T_j
+        double p00 = 0.0, p01 = 0.0, p11 = 0.0;
+        for (int j = 0; j < N; ++j) {
+            const LayerNum n = layer_numerators(lay + j * LAYER_STRIDE, k, c2, ic2);
+            const double id = 1.0 / n.Dh;
+            const double A = n.n00 * id, Bn = n.n01 * id, Dd = n.n11 * id;
+            const double E = n.ce * id, F = n.cf * id, G = n.cg * id;
+            ws(j, 4) = p00;
+            ws(j, 5) = p01;
+            ws(j, 6) = p11;
+            ws(j, 7) = A;
+            ws(j, 8) = Bn;
+            ws(j, 9) = Dd;
+            ws(j, 10) = E;
+            ws(j, 11) = F;
+            ws(j, 12) = G;
+            const double s00 = p00 + A, s01 = p01 + Bn, s11 = p11 + Dd;
+            const double is = 1.0 / fma(s00, s11, -s01 * s01);
+            // T = S^-1 [[E, F], [-F, G]];  P' = K22 - [[E, -F], [F, G]] T
+            const double t00 = fma(s11, E, s01 * F) * is, t01 = fma(s11, F, -s01 * G) * is;
+            const double t10 = -fma(s01, E, s00 * F) * is, t11 = fma(s00, G, -s01 * F) * is;
+            ws(j, 0) = t00;
+            ws(j, 1) = t01;
+            ws(j, 2) = t10;
+            ws(j, 3) = t11;
+            p00 = A - fma(E, t00, -F * t10);
+            p01 = -Bn - fma(E, t01, -F * t11);
+            p11 = Dd - fma(F, t01, G * t11);
+        }
+        // bottom-up: B_j, Q_j, and the most singular condensed block
+        const HalfNum hn = halfspace_numerators(lay + N * LAYER_STRIDE, c2);
+        const double iden = 1.0 / hn.den;
+        double b00 = hn.m00 * iden, b01 = hn.m01 * iden, b11 = hn.m11 * iden;
+        int js = N;
+        double g00 = p00 + b00, g01 = p01 + b01, g11 = p11 + b11;
+        double sn = fabs(fma(g00, g11, -g01 * g01));
+        double nrm = fma(g00, g00, fma(g11, g11, 2.0 * g01 * g01));
+        for (int j = N - 1; j >= 0; --j) {
+            const double A = ws(j, 7), Bn = ws(j, 8), Dd = ws(j, 9);
+            const double E = ws(j, 10), F = ws(j, 11), G = ws(j, 12);
+            const double m00 = b00 + A, m01 = b01 - Bn, m11 = b11 + Dd;
+            const double im = 1.0 / fma(m00, m11, -m01 * m01);
+            // Q = M^-1 [[E, -F], [F, G]];  B = K11 - [[E, F], [-F, G]] Q
+            const double q00 = fma(m11, E, -m01 * F) * im, q01 = -fma(m11, F, m01 * G) * im;
+            const double q10 = fma(m00, F, -m01 * E) * im, q11 = fma(m00, G, m01 * F) * im;
+            ws(j, 7) = q00;
+            ws(j, 8) = q01;
+            ws(j, 9) = q10;
+            ws(j, 10) = q11;
+            b00 = A - fma(E, q00, F * q10);
+            b01 = Bn - fma(E, q01, F * q11);
+            b11 = Dd - fma(-F, q01, G * q11);
+            const double h00 = ws(j, 4) + b00, h01 = ws(j, 5) + b01, h11 = ws(j, 6) + b11;
+            const double hs = fabs(fma(h00, h11, -h01 * h01));
+            const double hnrm = fma(h00, h00, fma(h11, h11, 2.0 * h01 * h01));
+            if (hs * nrm < sn * hnrm) {  // more singular: |det| / norm^2 smaller
+                js = j;
+                sn = hs;
+                nrm = hnrm;
+                g00 = h00;
+                g01 = h01;
+                g11 = h11;
+            }
+        }
+        // null vector of G from its larger row
+        double nx, nz;
+        if (fabs(g00) >= fabs(g11)) { nx = -g01; nz = g00; }
+        else { nx = -g11; nz = g01; }
+        const double nn = fmax(fabs(nx), fabs(nz));
+        nx /= nn;
+        nz /= nn;
+        // implicit-function rule, u propagated upward from js ...
+        double den = 0.0;
+        double x = nx, z = nz;
+        for (int j = js - 1; j >= 0; --j) {  // u_j = -T_j u_{j+1}
+            const double t00 = ws(j, 0), t01 = ws(j, 1), t10 = ws(j, 2), t11 = ws(j, 3);
+            const double x0 = -fma(t00, x, t01 * z), z0 = -fma(t10, x, t11 * z);
+            double qc, qb, qh;
+            elem_quad_grad(lay + j * LAYER_STRIDE, k, c, c2, x0, z0, x, z, &qc, &qb, &qh);
+            den += qc;
+            ws(j, 0) = qb;
+            ws(j, 1) = qh;
+            x = x0;
+            z = z0;
+        }
+        x = nx;  // ... and downward: u_{j+1} = -Q_j u_j
+        z = nz;
+        for (int j = js; j < N; ++j) {
+            const double q00 = ws(j, 7), q01 = ws(j, 8), q10 = ws(j, 9), q11 = ws(j, 10);
+            const double x1 = -fma(q00, x, q01 * z), z1 = -fma(q10, x, q11 * z);
+            double qc, qb, qh;
+            elem_quad_grad(lay + j * LAYER_STRIDE, k, c, c2, x, z, x1, z1, &qc, &qb, &qh);
+            den += qc;
+            ws(j, 0) = qb;
+            ws(j, 1) = qh;
+            x = x1;
+            z = z1;
+        }
+        const HalfD H = halfspace_d(lay + N * LAYER_STRIDE, c);
+        const D4 qhs = half_quad(H, x, z);
+        den += qhs.d0;
+        const double inv = -1.0 / den;
+        row[N] = qhs.d1 * inv;
+        for (int j = 0; j < N; ++j) {
+            row[j] = ws(j, 0) * inv;
+            row[N + 1 + j] = ws(j, 1) * inv;
+        }
     }
-    const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
-    double k = b.k[it];
-    double c2 = c * c;
-    // node j slot: [0..3] S_j (top-down), [4..7] M_j = B_{j+1} + K22_j,
-    //              [8..11] B_j (bottom-up), [12..15] P_j,
-    //              [16..21] layer j's element entries (A, B, Dd, E, F, G)
-    M2 P = {0.0, 0.0, 0.0, 0.0};
-    for (int j = 0; j < N; ++j) {
-        M2 K11, K12, K21, K22;
-        elem_blocks(lay + j * LAYER_STRIDE, k, c2, &K11, &K12, &K21, &K22);
-        double* E6 = ws + 24 * j + 16;
-        E6[0] = K11.a; E6[1] = K11.b; E6[2] = K11.d; E6[3] = K12.a; E6[4] = K12.b; E6[5] = K12.d;
-        M2 S = madd(P, K11);
-        st(ws + 24 * j, S);
-        st(ws + 24 * j + 12, P);
-        P = msub(K22, mmul(K21, msolve(S, K12)));
-    }
-    st(ws + 24 * N + 12, P);
-    HalfNum hn = halfspace_numerators(lay + N * LAYER_STRIDE, c2);
-    double iden = 1.0 / hn.den;
-    M2 Bv = {hn.m00 * iden, hn.m01 * iden, hn.m01 * iden, hn.m11 * iden};
-    st(ws + 24 * N + 8, Bv);
-    for (int j = N - 1; j >= 0; --j) {
-        M2 K11, K12, K21, K22;
-        stored_blocks(ws + 24 * j + 16, &K11, &K12, &K21, &K22);
-        M2 Mj = madd(Bv, K22);
-        st(ws + 24 * j + 4, Mj);
-        Bv = msub(K11, mmul(K12, msolve(Mj, K21)));
-        st(ws + 24 * j + 8, Bv);
-    }
-    // twist node: most singular condensed block
-    int js = N;
-    double best = 1e300;
-    for (int j = 0; j <= N; ++j) {
-        M2 Pj, Bj;
-        ld(ws + 24 * j + 12, &Pj);
-        ld(ws + 24 * j + 8, &Bj);
-        M2 G = madd(Pj, Bj);
-        double nrm = G.a * G.a + G.b * G.b + G.c * G.c + G.d * G.d;
-        double sng = fabs(mdet(G)) / nrm;
-        if (sng < best) { best = sng; js = j; }
-    }
-    M2 G;
-    {
-        M2 Pj, Bj;
-        ld(ws + 24 * js + 12, &Pj);
-        ld(ws + 24 * js + 8, &Bj);
-        G = madd(Pj, Bj);
-    }
-    // null vector of the 2x2 G from its larger row
-    double nx, nz;
-    if (G.a * G.a + G.b * G.b >= G.c * G.c + G.d * G.d) { nx = -G.b; nz = G.a; }
-    else { nx = -G.d; nz = G.c; }
-    double nn = fmax(fabs(nx), fabs(nz));
-    nx /= nn; nz /= nn;
-    // store u_j in the P slot (no longer needed): [12], [13]
-    ws[24 * js + 12] = nx;
-    ws[24 * js + 13] = nz;
-    for (int j = js - 1; j >= 0; --j) {  // upward: u_j = -S_j^-1 K12_j u_{j+1}
-        M2 K11, K12, K21, K22, S;
-        stored_blocks(ws + 24 * j + 16, &K11, &K12, &K21, &K22);
-        ld(ws + 24 * j, &S);
-        double x = ws[24 * (j + 1) + 12], z = ws[24 * (j + 1) + 13];
-        double v0 = K12.a * x + K12.b * z, v1 = K12.c * x + K12.d * z, o0, o1;
-        mvsolve(S, v0, v1, &o0, &o1);
-        ws[24 * j + 12] = -o0;
-        ws[24 * j + 13] = -o1;
-    }
-    for (int j = js + 1; j <= N; ++j) {  // downward: u_j = -M_{j-1}^-1 K21_{j-1} u_{j-1}
-        M2 K11, K12, K21, K22, Mj;
-        stored_blocks(ws + 24 * (j - 1) + 16, &K11, &K12, &K21, &K22);
-        ld(ws + 24 * (j - 1) + 4, &Mj);
-        double x = ws[24 * (j - 1) + 12], z = ws[24 * (j - 1) + 13];
-        double v0 = K21.a * x + K21.b * z, v1 = K21.c * x + K21.d * z, o0, o1;
-        mvsolve(Mj, v0, v1, &o0, &o1);
-        ws[24 * j + 12] = -o0;
-        ws[24 * j + 13] = -o1;
-    }
-    // implicit-function rule with dual-number element derivatives
-    HalfD H = halfspace_d(lay + N * LAYER_STRIDE, c);
-    D4 qh = half_quad(H, ws[24 * N + 12], ws[24 * N + 13]);
-    double den = qh.d0;
-    row[N] = qh.d1;
-    for (int j = 0; j < N; ++j) {
-        ElemD K = layer_element_d(lay + j * LAYER_STRIDE, k, c);
-        D4 q = elem_quad(K, ws[24 * j + 12], ws[24 * j + 13], ws[24 * (j + 1) + 12],
-                         ws[24 * (j + 1) + 13]);
-        den += q.d0;
-        row[j] = q.d1;
-        row[N + 1 + j] = q.d2;
-    }
-    double inv = -1.0 / den;
-    for (int p = 0; p < 2 * N + 1; ++p) row[p] *= inv;
 }
 
-cudaError_t launch_root_grad(const DevBatch& b, const double* croot, double* rows, double* bs,
-                             cudaStream_t s) {
+// Threads of root_grad_kernel for n_items items: at most 256 per SM (the FP64
+// pipe is busy with fewer), so that the scratch of models of up to 23 layers
+// stays within the 129 MB L2.
+static int root_grad_threads(int n_items, int sms) {
+    const int most = 256 * (sms > 0 ? sms : 152);
+    return std::max(ROOT_THREADS, std::min(most, (n_items + ROOT_THREADS - 1) / ROOT_THREADS * ROOT_THREADS));
+}
+size_t root_grad_scratch(int n_items, int max_layers, int sms) {
+    return (size_t)root_grad_threads(n_items, sms) * ROOT_SLOTS * std::max(max_layers, 1);
+}
+
+cudaError_t launch_root_grad(const DevBatch& b, const double* croot, double* rows, double* scratch,
+                             int sms, cudaStream_t s) {
     if (b.n_items <= 0) return cudaSuccess;
-    root_grad_kernel<<<(b.n_items + 63) / 64, 64, 0, s>>>(b, croot, rows, bs);
+    root_grad_kernel<<<root_grad_threads(b.n_items, sms) / ROOT_THREADS, ROOT_THREADS, 0, s>>>(
+        b, croot, rows, scratch);
     return cudaGetLastError();
 }
 
