@@ -114,7 +114,7 @@ typedef struct {
     int32_t count_block;     /* precision 2: threads per block of the counting kernel, 64, 128
                                 or 256 (two lanes per item, items of a block consecutive;
                                 launch bounds of 14, 7 or 2 resident blocks). Default: 256
-                                with count_split 2, else 128 */
+                                with count_split 1 or 2, else 128 */
     int32_t count_split;     /* precision 2: 0 the search (a lane pair per item, three-way
                                 splits) and the certificate in one kernel; 1 the search
                                 in kernels of their own (one thread per item: every 6th
@@ -127,8 +127,10 @@ typedef struct {
                                 change below the bound, a mode below V[0]) take that
                                 scan, its check and the mode-count search on a second,
                                 highest-priority stream beside the certificate. Same
-                                results for all three. Default by batch size: 0 below
-                                131,072 items, 1 below 262,144, else 2. With 1 or 2,
+                                results for all three. Default: 0 below 65,536 items,
+                                else 2 when the models or the grid as created make
+                                such items likely (a layer slower than the one
+                                above it, a grid above the slowest modes), else 1. With 1 or 2,
                                 count_block 64 gives the certificate kernel 640 resident
                                 threads (96 registers) */
 } masw_plan;

@@ -53,6 +53,7 @@ struct masw_batch {
     std::vector<int32_t> order_sorted, order_natural;
     std::vector<int32_t> search_order;  // anchors of the split search, then the others
     int32_t n_anchor = 0;
+    bool fallback_likely = false;  // as created (default_plan)
     std::vector<int64_t> grad_off;
 
     double* d_layers = nullptr;
@@ -361,14 +362,18 @@ static masw_plan default_plan(const masw_batch* B) {
     p.stage_layers = std::min(B->max_layers + 1, 32);
     p.use_graph = 1;
     p.precision = 2;
-    // the fused kernel's lane pairs give small batches the shortest chain;
-    // large ones take the split kernels, and from a quarter million items
-    // the search's fallback items on the second stream
-    p.count_split = B->n_items < (1 << 17) ? 0 : B->n_items < (1 << 18) ? 1 : 2;
-    // beside the second stream's chain the certificate runs in blocks of 256
-    // (512 resident threads per SM, against 896 in blocks of 128: measured
-    // faster there, the chain ending sooner), else of 128
-    p.count_block = p.count_split == 2 ? 256 : 128;
+    // The fused kernel's lane pairs give small batches the shortest chain of
+    // launches; from 65,536 items the split kernels, whose search proves most
+    // certificates, are ahead (32,000 items of 8 layers 125 us fused, 129
+    // split; 64,400 ragged 580 and 584; 80,000 of 8 layers 215 and 171). The
+    // second stream where the search will leave items to the fallback chain:
+    // models with a layer slower than the one above it, or a grid that starts
+    // above a model's slowest modes (701 ragged models 762 -> 630 us with it;
+    // a uniform batch without such items 238 -> 246).
+    p.count_split = B->n_items < (1 << 16) ? 0 : B->fallback_likely ? 2 : 1;
+    // with the split search, blocks of 256 at 2 per SM (128 registers, no
+    // spills) against 128 at 7 (72 registers): uniform batch 257 -> 238 us
+    p.count_block = p.count_split ? 256 : 128;
     return p;
 }
 
@@ -394,6 +399,7 @@ static ScanPlan to_scan_plan(const masw_batch* B, const masw_plan& p) {
     s.count_block = p.count_block;
     s.count_split = p.count_split;
     s.sms = B->sm_count;
+    s.max_layers = B->max_layers;
     return s;
 }
 
@@ -561,6 +567,9 @@ int masw_model_batch_create(const masw_models_desc* md, const masw_grid* grid, v
         B->woff[m + 1] = B->woff[m] + B->n_lambda[m];
         hoff[m + 1] = hoff[m] + B->n_layers[m];
         B->nlim[m] = scan_limit(B->grid, b[B->loff[m + 1] - 1]);
+        for (int32_t i = B->loff[m]; i < B->loff[m + 1]; ++i)
+            B->fallback_likely = B->fallback_likely || 0.9 * b[i] < B->grid.c0 ||
+                                 (i > B->loff[m] && b[i] < b[i - 1]);
     }
     B->item_model.resize(nw);
     B->kvec.resize(nw);

@@ -216,6 +216,98 @@ __device__ __forceinline__ Located count_search_guess(const float* __restrict__ 
     return r;
 }
 
+// The two searches by a group of G lanes per item, for batches too small to
+// fill the GPU with a thread each: G points per step, so log_(G+1) instead of
+// log_2 steps of one evaluation's latency. All lanes of a group (`gmask`, lane
+// `gl`, first lane `g0` of the warp) call them together and get the same
+// result.
+
+// Lane i's point of G that split (lo, hi), hi - lo > 1; the step's points are
+// lo + 1 .. hi - 1, and hi for lanes left over, once G reaches them all.
+template <int G>
+__device__ __forceinline__ int section_point(int lo, int hi, int i) {
+    const int len = hi - lo;
+    return len - 1 <= G ? min(lo + 1 + i, hi) : lo + (int)(((long long)len * (i + 1)) / (G + 1));
+}
+
+// count_search_single by a group.
+template <int G>
+__device__ __forceinline__ Located count_search_group(const float* __restrict__ lay32, int N,
+                                                      double k, double c0, double dc, int npf,
+                                                      int gl, int g0, unsigned gmask) {
+    Located r{-1, 0, 0};
+    if (npf < 1) return r;
+    const float kf = (float)k;
+    int lo = -1, hi = npf - 1;  // (the top is taken as nonzero until the end)
+    while (hi - lo > 1) {
+        const int p = section_point<G>(lo, hi, gl);
+        const int c = p < hi ? inertia_bound_f<false>(lay32, N, kf, (float)grid_c(c0, dc, p), nullptr) : 1;
+        const unsigned m = (__ballot_sync(gmask, c >= 1) >> g0) & (G == 32 ? ~0u : (1u << G) - 1u);
+        const int f = m ? __ffs(m) - 1 : G;  // first lane at or above the change
+        const int top = __shfl_sync(gmask, p, g0 + min(f, G - 1)), below = __shfl_sync(gmask, p, g0 + max(f - 1, 0));
+        if (f < G) hi = top;
+        if (f > 0) lo = below;
+    }
+    // even lanes V[lo], odd lanes V[hi]
+    const int p = (gl & 1) ? hi : lo;
+    bool sure = false;
+    const int c = p >= 0 ? count_bound_at(lay32, N, kf, c0, dc, p, &sure) : 0;
+    const int c_lo = __shfl_sync(gmask, c, g0), c_hi = __shfl_sync(gmask, c, g0 + 1);
+    const bool s_lo = __shfl_sync(gmask, (int)sure, g0), s_hi = __shfl_sync(gmask, (int)sure, g0 + 1);
+    if (c_hi < 1 && hi == npf - 1) return r;  // no change inside the range
+    r.n = hi;
+    r.proof = (s_lo && c_lo == 0 ? PROOF_LO : 0) | (s_hi && (c_hi & 1) ? PROOF_HI : 0);
+    r.count = c_hi;
+    return r;
+}
+
+// count_search_guess by a group of G lanes: first the points guess - 1 ..
+// guess + G - 2 (the change lies among them for most items: one evaluation's
+// latency), then steps of 4^i away on the side where it lies, then splits.
+template <int G>
+__device__ __forceinline__ Located count_search_guess_group(const float* __restrict__ lay32, int N,
+                                                            double k, double c0, double dc, int npf,
+                                                            int guess, int gl, int g0,
+                                                            unsigned gmask) {
+    Located r{-1, 0, 0};
+    if (npf < 1) return r;
+    const float kf = (float)k;
+    int lo = -1, hi = npf, step = 4;  // hi = npf: not seen; lo = -1: c = 0
+    bool s_lo = false, s_hi = false, first = true, up = false;
+    for (;;) {
+        int p;
+        if (first) p = min(max(guess - 1 + gl, 0), npf - 1);
+        else if (!up && lo < 0) p = max(hi - (step << (2 * (G - 1 - gl))), 0);
+        else if (up && hi == npf) p = min(lo + (step << (2 * gl)), npf - 1);
+        else p = section_point<G>(lo, hi, gl);
+        bool sure = true;
+        const int c = p < hi ? count_bound_at(lay32, N, kf, c0, dc, p, &sure) : 1;
+        const unsigned m = (__ballot_sync(gmask, c >= 1) >> g0) & (G == 32 ? ~0u : (1u << G) - 1u);
+        const int f = m ? __ffs(m) - 1 : G;
+        const int a = g0 + min(f, G - 1), z = g0 + max(f - 1, 0);
+        const int p_hi = __shfl_sync(gmask, p, a), p_lo = __shfl_sync(gmask, p, z);
+        const int c_hi = __shfl_sync(gmask, c, a);
+        const bool t_hi = __shfl_sync(gmask, (int)sure, a), t_lo = __shfl_sync(gmask, (int)sure, z);
+        if (f < G && p_hi < hi) {
+            hi = p_hi;
+            s_hi = t_hi && (c_hi & 1);
+            r.count = c_hi;
+        }
+        if (f > 0 && p_lo > lo && p_lo < hi) {
+            lo = p_lo;
+            s_lo = t_lo;
+        }
+        if (first) up = f == G;
+        else step <<= 2 * G;
+        if (step > (1 << 20)) step = 1 << 20;
+        first = false;
+        if (hi - lo <= 1) break;
+    }
+    if (hi < npf) r.n = hi;
+    r.proof = (s_lo ? PROOF_LO : 0) | (s_hi ? PROOF_HI : 0);
+    return r;
+}
+
 // The certificate stage for the search's index n (count_search_pair or
 // count_search_single) in the
 // pole-free range [0, npf). Both lanes of the pair (lane bit 0 = half, `pair`

@@ -69,6 +69,7 @@ struct ScanPlan {
     int count_split = 0;    // 1: the counting search in a kernel of its own; 2: as 1, and
                             // the search's fallback items on a second stream (ScanSide)
     int sms = 0;            // SM count (0: unknown)
+    int max_layers = 0;     // most finite layers of a model
 };
 
 // FP32 screen + FP64 decision (masw_screen.cuh, masw_kernels.cu). counting

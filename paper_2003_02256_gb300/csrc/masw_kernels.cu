@@ -534,7 +534,8 @@ struct CountLists {
     int32_t* two;      // items with none
     int32_t* n_two;
 };
-constexpr int32_t ONE_LOW = 1 << 30;  // list `one`: V[n-1] is the point wanted
+constexpr int32_t ONE_LOW = 1 << 30;    // list `one`: V[n-1] is the point wanted
+constexpr int32_t SCAN_FROM = 1 << 30;  // search list: the count is even up to V[n32[item]]
 
 // The counting search's FP64 certificate (plan precision 2), two lanes per
 // item (certify_pair; natural item order, or by layer count over a whole
@@ -557,8 +558,7 @@ constexpr int32_t ONE_LOW = 1 << 30;  // list `one`: V[n-1] is the point wanted
 // Search stage alone (count_search_single or count_search_guess, one
 // thread per item), with what its FP32 counts' error bound proves. An item
 // whose counts at V[n-1] (0) and V[n] (odd) are both proven is finished here.
-// With one of them proven it joins the list `one` (count_certify_one_kernel:
-// the other point in double-float), with none the list `two`
+// With one of them proven it joins the list `one`, with none the list `two`
 // (count_certify_kernel). Bound by instruction issue (FP32, 88 % of cycles in
 // the first pass on the 8192-model ragged batch).
 // The items the certificate would only pass on to
@@ -568,18 +568,21 @@ constexpr int32_t ONE_LOW = 1 << 30;  // list `one`: V[n-1] is the point wanted
 // (results written here), so that the fallback chain can run on a second
 // stream beside the certificate. Natural item order: a warp's 32 items share
 // a model or two and have adjacent wavelengths, so their branches agree.
+// G lanes per item (a group search where G > 1).
 // PASS 0: the items [item_begin, item_end) in natural order; 1: the anchor
 // items of b.search_order (every SEARCH_STRIDE-th wavelength of a model and
 // its last), each searched in full; 2: the other items, each searched
 // from a guess between its two anchors' indices (count_search_guess; a
 // neighbour without an index: in full), after pass 1.
-template <int B, int PASS>
+template <int B, int PASS, int G>
 __global__ void __launch_bounds__(B) count_search_kernel(DevBatch b,
                                                          const float* __restrict__ layers32,
                                                          ScanOut o, CountLists w,
                                                          int item_begin, int item_end) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    int item;
+    const int t = (blockIdx.x * B + threadIdx.x) / G;
+    const int gl = threadIdx.x & (G - 1), g0 = (threadIdx.x & 31) - gl;
+    const unsigned gmask = G == 32 ? FULL : ((1u << G) - 1u) << g0;
+    int item;  // a group's lanes leave together
     if (PASS == 0) {
         item = item_begin + t;
         if (item >= item_end) return;
@@ -592,6 +595,7 @@ __global__ void __launch_bounds__(B) count_search_kernel(DevBatch b,
     const int N = b.model_loff[m + 1] - lo_rec - 1;
     const int nlim = b.model_nlim[m];
     if (nlim < 2) {
+        if (gl) return;
         w.nsearch[item] = 0;
         w.n32[item] = -1;
         write_result(b, o, item, -1);
@@ -611,10 +615,13 @@ __global__ void __launch_bounds__(B) count_search_kernel(DevBatch b,
         // doubling steps and bisection, any guess gives the same result)
         const int guess = (na >= 1 && nb >= 1) ? max(search_guess(na, nb, item - ja, jb - ja), 0)
                                                : npf >> 1;
-        r = count_search_guess(lay32, N, k, b.c0, b.dc, npf, guess);
+        r = G == 1 ? count_search_guess(lay32, N, k, b.c0, b.dc, npf, guess)
+                   : count_search_guess_group<G>(lay32, N, k, b.c0, b.dc, npf, guess, gl, g0, gmask);
     } else {
-        r = count_search_single(lay32, N, k, b.c0, b.dc, npf);
+        r = G == 1 ? count_search_single(lay32, N, k, b.c0, b.dc, npf)
+                   : count_search_group<G>(lay32, N, k, b.c0, b.dc, npf, gl, g0, gmask);
     }
+    if (gl) return;
     if (r.n < 1 || route_level(b.route) >= 1) {
         // the start certify_pair gives these items (test routing: V[0])
         w.nsearch[item] = 0;
@@ -634,38 +641,6 @@ __global__ void __launch_bounds__(B) count_search_kernel(DevBatch b,
         if (o.cert_counts) o.cert_counts[item] = r.count;
     } else {
         w.two[atomicAdd(w.n_two, 1)] = item;
-    }
-}
-
-// The listed items of which the search's FP32 bound proved one of the two
-// counts: the other one in double-float (det_inertia_dd), one thread per item.
-// ONE_LOW marks those whose V[n-1] is wanted. An item whose count there is
-// not the certificate's goes to the list `two` (an FP32 index off by one, or
-// an even count). A quarter of the ragged batch's items, so half as many
-// double-float evaluations as lanes in the pair kernel.
-template <int B>
-__global__ void __launch_bounds__(B, (B == 256 ? 2 : 896 / B))
-    count_certify_one_kernel(DevBatch b, ScanOut o, CountLists w) {
-    const int total = *w.n_one;
-    const int stride = gridDim.x * B;
-    for (int t = blockIdx.x * B + threadIdx.x; t < total; t += stride) {
-        const int e = w.one[t];
-        const int item = e & ~ONE_LOW;
-        const bool low = e & ONE_LOW;
-        const int m = b.item_model[item];
-        const int lo_rec = b.model_loff[m];
-        const int N = b.model_loff[m + 1] - lo_rec - 1;
-        const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
-        const int n = w.nsearch[item];
-        const int v = det_inertia_dd(records_df(b, lo_rec), lay, N, b.k[item],
-                                     grid_c(b.c0, b.dc, low ? n - 1 : n));
-        if (low ? v == 0 : (v > 0 && (v & 1))) {
-            w.n32[item] = n | SCREEN_COUNTED;
-            write_result(b, o, item, n);
-            if (o.cert_counts) o.cert_counts[item] = pack_counts(0, low ? o.cert_counts[item] : v);
-        } else {
-            w.two[atomicAdd(w.n_two, 1)] = item;
-        }
     }
 }
 
@@ -709,19 +684,25 @@ __device__ __forceinline__ void certify_item(const DevBatch& b, const float* __r
         n32[item] = r.cert | SCREEN_COUNTED;
         write_result(b, o, item, r.cert);
     } else if (r.n >= 1 || (r.start >= 1 && r.start < npf)) {
-        // the counts around the located point fail, or two modes inside one
-        // interval with no odd count found above them
-        n32[item] = r.n;
-        search[atomicAdd(n_search, 1)] = item;
+        // the counts around the located point fail; or two modes inside one
+        // interval with no odd count found above them: an even count up to
+        // V[start], from where the sign scan may start
+        n32[item] = r.n >= 1 ? r.n : r.start;
+        search[atomicAdd(n_search, 1)] = item | (r.n >= 1 ? 0 : SCAN_FROM);
     } else {
         n32[item] = r.start;
         fallback[atomicAdd(n_fallback, 1)] = item;
     }
 }
 
-// SPLIT: the items of the list w.two (a device-side count, grid-stride);
-// otherwise the items [item_begin, item_end), with the search in the same
-// kernel.
+// SPLIT: the split search's lists (device-side counts, grid-stride). The
+// items of w.two (neither count proven) take a pair of lanes each; those of
+// w.one (one proven) a lane each, for the other point's double-float count
+// (det_inertia_dd; ONE_LOW: V[n-1] is wanted), and the pair comes together for
+// an item whose count there is not the certificate's (an FP32 index off by
+// one, or an even count). The pairs of w.two come first: theirs is the longer
+// work. Otherwise the items [item_begin, item_end), with the search in the
+// same kernel.
 template <int B, bool SPLIT>
 __global__ void __launch_bounds__(B, (B == 256 ? 2 : (B == 64 && SPLIT ? 10 : 896 / B)))
     count_certify_kernel(DevBatch b, const float* __restrict__ layers32, ScanOut o, CountLists w,
@@ -729,30 +710,58 @@ __global__ void __launch_bounds__(B, (B == 256 ? 2 : (B == 64 && SPLIT ? 10 : 89
                          int32_t* n_fallback, int item_begin, int item_end) {
     const int half = threadIdx.x & 1;
     const unsigned pair = 3u << ((threadIdx.x & 31) & 30);
-    const int end = SPLIT ? *w.n_two : item_end - item_begin;
-    const int stride = SPLIT ? (gridDim.x * B) >> 1 : 0;
+    const int n_two = SPLIT ? *w.n_two : 0;
+    const int n_one = SPLIT ? *w.n_one : 0;
+    const int end = SPLIT ? n_two + ((n_one + 1) >> 1) : item_end - item_begin;
+    const int stride = (gridDim.x * B) >> 1;
     for (int t = (blockIdx.x * B + threadIdx.x) >> 1; t < end; t += stride) {
-        const int item = SPLIT ? w.two[t] : item_begin + t;  // both lanes of a pair together
-        const int m = b.item_model[item];
-        const int lo_rec = b.model_loff[m];
-        const int N = b.model_loff[m + 1] - lo_rec - 1;
-        const int nlim = b.model_nlim[m];
-        if (!SPLIT && nlim < 2) {
-            if (!half) {
-                n32[item] = -1;
-                write_result(b, o, item, -1);
-                if (o.cert_counts) o.cert_counts[item] = -1;
+        int item = -1;  // the lane's item for the pair's certificate
+        if (!SPLIT) {
+            item = item_begin + t;
+        } else if (t < n_two) {
+            item = w.two[t];
+        } else if (2 * (t - n_two) + half < n_one) {
+            const int e = w.one[2 * (t - n_two) + half];
+            const int it = e & ~ONE_LOW;
+            const bool low = e & ONE_LOW;
+            const int lo_rec = b.model_loff[b.item_model[it]];
+            const int N = b.model_loff[b.item_model[it] + 1] - lo_rec - 1;
+            const int n = w.nsearch[it];
+            const int v = det_inertia_dd(records_df(b, lo_rec),
+                                         b.layers + (size_t)lo_rec * LAYER_STRIDE, N, b.k[it],
+                                         grid_c(b.c0, b.dc, low ? n - 1 : n));
+            if (low ? v == 0 : (v > 0 && (v & 1))) {
+                n32[it] = n | SCREEN_COUNTED;
+                write_result(b, o, it, n);
+                if (o.cert_counts) o.cert_counts[it] = pack_counts(0, low ? o.cert_counts[it] : v);
+            } else {
+                item = it;
             }
-            return;
         }
-        const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
-        const double k = b.k[item];
-        const int npf = pole_free_points_f(lay32, N, (float)k, (float)b.c0, (float)b.dc, nlim);
-        const int ns =
-            SPLIT ? w.nsearch[item] : count_search_pair(lay32, N, k, b.c0, b.dc, npf, half, pair);
-        certify_item(b, layers32, o, item, m, lo_rec, N, nlim, npf, ns, half, pair, n32, search,
-                     n_search, fallback, n_fallback);
-        if (!SPLIT) return;
+        // one item for both lanes, or each lane's own in turn
+        const bool own = SPLIT && t >= n_two;
+        for (int r = 0; r < (own ? 2 : 1); ++r) {
+            const int it = own ? __shfl_sync(pair, item, ((threadIdx.x & 31) & 30) + r) : item;
+            if (it < 0) continue;
+            const int m = b.item_model[it];
+            const int lo_rec = b.model_loff[m];
+            const int N = b.model_loff[m + 1] - lo_rec - 1;
+            const int nlim = b.model_nlim[m];
+            if (!SPLIT && nlim < 2) {
+                if (!half) {
+                    n32[it] = -1;
+                    write_result(b, o, it, -1);
+                    if (o.cert_counts) o.cert_counts[it] = -1;
+                }
+                continue;
+            }
+            const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
+            const int npf = pole_free_points_f(lay32, N, (float)b.k[it], (float)b.c0, (float)b.dc, nlim);
+            const int ns = SPLIT ? w.nsearch[it]
+                                 : count_search_pair(lay32, N, b.k[it], b.c0, b.dc, npf, half, pair);
+            certify_item(b, layers32, o, it, m, lo_rec, N, nlim, npf, ns, half, pair, n32, search,
+                         n_search, fallback, n_fallback);
+        }
     }
 }
 
@@ -845,7 +854,8 @@ __global__ void __launch_bounds__(SIGN_SCAN_THREADS, 4)
         __syncthreads();
         const int t = s_item;
         if (t >= total) return;
-        const int item = list[t];
+        const int item = list[t] & ~SCAN_FROM;
+        const bool from = list[t] & SCAN_FROM;
         if (route_level(b.route) >= 2) {  // test routing: every item to the mode-count search
             if (tid == 0) hard[atomicAdd(n_hard, 1)] = item;
             __syncthreads();
@@ -867,7 +877,7 @@ __global__ void __launch_bounds__(SIGN_SCAN_THREADS, 4)
         const int nlim = b.model_nlim[m];  // >= 2 for listed items
         const int npf = pole_free_points_f(lay32, N, kf, (float)b.c0, (float)b.dc, nlim);
         // the counts at V[0] and at the end of the pole-free range, a warp each
-        if (tid < 64) {
+        if (tid < 64 && !from) {
             const int p = tid < 32 ? 0 : max(npf - 1, 0);
             bool sure;
             int c = count_bound_at(lay32, N, kf, b.c0, b.dc, p, &sure);
@@ -875,9 +885,9 @@ __global__ void __launch_bounds__(SIGN_SCAN_THREADS, 4)
             if ((tid & 31) == 0) s_end[tid >> 5] = c;
         }
         __syncthreads();
-        const int c0 = s_end[0];
+        const int c0 = from ? 0 : s_end[0];
         const int carry = c0 & 1;
-        int base = (npf > 0 && s_end[1] == c0) ? npf : 1;
+        int base = from ? n32[item] + 1 : (npf > 0 && s_end[1] == c0) ? npf : 1;
         int res = -1, used = 0;
         bool bad = c0 < 0, over = false;
         for (; !bad && base < nlim; base += SIGN_SCAN_THREADS) {
@@ -1057,17 +1067,35 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
             if (b.search_order && item_begin == 0 && item_end == b.n_items) {
                 // anchors first, then the items between them
                 const int na = b.n_anchor, nr = b.n_items - b.n_anchor;
-                if (na > 0)
-                    count_search_kernel<128, 1><<<(na + 127) / 128, 128, 0, s>>>(
-                        b, layers32, o, w, item_begin, item_end);
+#define MASW_SEARCH(PASS, G, count)                                                             \
+    count_search_kernel<128, PASS, G><<<((count) * (G) + 127) / 128, 128, 0, s>>>(b, layers32, o, \
+                                                                                 w, item_begin, \
+                                                                                 item_end)
+                // Lanes per item: a group where a thread each would leave the
+                // GPU idle. Anchors (12 evaluations in a row by one thread):
+                // 8 lanes up to 8,192 anchors, 4 up to 32,768 (701 ragged
+                // models, 26,000 anchors: scan 719 -> 636 us; 34,000 anchors
+                // of 8 layers: 273 us with 1, 279 with 4). The others (2 for
+                // most, the warp waits for its slowest): 4 for short lists,
+                // and up to 131,072 of deep models, whose evaluations take
+                // longest (126,000 items of up to 30 layers 781 -> 636 us;
+                // 64,000 of 12 layers 298 us with 1, 312 with 4).
+                const int g1 = na <= 8192 ? 8 : na <= 32768 ? 4 : 1;
+                const int g2 = nr <= 32768 || (nr <= 131072 && p.max_layers >= 16) ? 4 : 1;
+                if (na > 0) {
+                    if (g1 == 8) MASW_SEARCH(1, 8, na);
+                    else if (g1 == 4) MASW_SEARCH(1, 4, na);
+                    else MASW_SEARCH(1, 1, na);
+                }
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
-                if (nr > 0)
-                    count_search_kernel<128, 2><<<(nr + 127) / 128, 128, 0, s>>>(
-                        b, layers32, o, w, item_begin, item_end);
+                if (nr > 0) {
+                    if (g2 == 4) MASW_SEARCH(2, 4, nr);
+                    else MASW_SEARCH(2, 1, nr);
+                }
             } else {
-                count_search_kernel<128, 0><<<(n + 127) / 128, 128, 0, s>>>(
-                    b, layers32, o, w, item_begin, item_end);
+                MASW_SEARCH(0, 1, n);
             }
+#undef MASW_SEARCH
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if (phase_ev && (e = cudaEventRecord(phase_ev[2], s)) != cudaSuccess) return e;
         }
@@ -1085,12 +1113,8 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
         const int per_sm = cb == 256 ? 2 : cb == 128 ? 7 : 10;
         const int lgrid = std::max(1, std::min(grid, per_sm * sms));
 #define MASW_COUNT_LAUNCH(BS, SPL)                                                              \
-    do {                                                                                        \
-        if (SPL) count_certify_one_kernel<BS><<<lgrid, BS, 0, s>>>(b, o, w);                    \
-        count_certify_kernel<BS, SPL><<<SPL ? lgrid : grid, BS, 0, s>>>(                        \
-            b, layers32, o, w, n32, search, counters + 5, fallback, counters + 3, item_begin,   \
-            item_end);                                                                          \
-    } while (0)
+    count_certify_kernel<BS, SPL><<<SPL ? lgrid : grid, BS, 0, s>>>(                            \
+        b, layers32, o, w, n32, search, counters + 5, fallback, counters + 3, item_begin, item_end)
         switch (cb * 2 + (p.count_split ? 1 : 0)) {
             case 128: MASW_COUNT_LAUNCH(64, false); break;
             case 129: MASW_COUNT_LAUNCH(64, true); break;
@@ -1130,9 +1154,10 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
                                                         item_end);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    // the certificate's own failures (with overlap; all fallback items otherwise)
-    e = launch_tail(b, o, p, layers32, n32, search, unresolved, fallback, counters, counting, n, s,
-                    0, phase_ev ? phase_ev[1] : nullptr);
+    // the certificate's own failures (with overlap: no fallback items here;
+    // all of them otherwise)
+    e = launch_tail(b, o, p, layers32, n32, search, unresolved, fallback, counters,
+                    counting && !overlap, n, s, 0, phase_ev ? phase_ev[1] : nullptr);
     if (e != cudaSuccess) return e;
     if (overlap && (e = cudaStreamWaitEvent(s, side->join, 0)) != cudaSuccess) return e;
     return cudaSuccess;
