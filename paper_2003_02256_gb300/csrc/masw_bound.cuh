@@ -3,53 +3,56 @@
 //
 // The certificate of the counting search needs the count at V[n-1] and V[n].
 // Its double-float recurrence takes about 1,640 thread instructions a
-// layer-evaluation, this one about 250, and the root lies anywhere between
+// layer-evaluation, this one about 280, and the root lies anywhere between
 // the two points: a relative distance of u dc / c from the nearer one, u
-// uniform, against FP32 errors of 1e-7 .. 1e-4 of the pivots. So most counts
+// uniform, against FP32 errors of 1e-7 .. 1e-5 of the pivots. So most counts
 // are already decided here, with a floating-point filter: the recurrence
-// carries a bound e on the spectral norm of the error of its 2x2 state P, a
-// pivot S = P + K11 whose error bound stays below half its smallest
-// eigenvalue has the inertia of the exact one, and when every pivot does, the
+// carries a bound E of the error of its 2x2 state P (-E <= error <= E, a
+// symmetric matrix), a pivot S = P + K11 whose bound keeps every perturbed S
+// nonsingular has the inertia of the exact one, and when every pivot does, the
 // count is the exact count of K (Sylvester). Otherwise the point goes to the
 // double-float recurrence (masw_df.cuh), which also decides whatever this
 // filter cannot.
 //
 // The recurrence. A layer thin next to the wavelength has K11, K12 of order
 // 1/(kh) and P' - P of order kh, so P' = K22 - K21 S^-1 K12 loses (kh)^-2 in
-// relative accuracy. With W = P + K11 + K12 (= S + K12) and R = S^-1 W the same
-// P' is
-//   P' = P + 2 diag(A + E, D + G) - W^T R
+// relative accuracy. With W = P + K11 + K12 (= S + K12) the same P' is
+//   P' = P + 2 diag(A + E, D + G) - W^T S^-1 W
 // (K11 = [[A, B], [B, D]], K12 = [[E, F], [-F, G]], K22 = [[A, -B], [-B, D]]),
 // whose terms are of order kh where A + E and D + G are formed without
-// cancellation: A + E from e^-x cosh x - e^-x = (1 - e^-x)^2 / 2.
+// cancellation: A + E from e^-x cosh x - e^-x = (1 - e^-x)^2 / 2. For a thick
+// layer K12 is the small one and the first form has no cancellation; the
+// smaller of W and K12 picks the form.
 //
 // The bound (first order, with the second-order factor of S^-1; eps = 2^-24).
-// With T = S^-1 K12 = R - I and ||T|| its 2-norm (from ||T||_F and det T), an
-// error e of P reaches P' as ||T||^2 e. The computed element differs from the
-// exact one in three ways:
+// With T = S^-1 K12 and R = S^-1 W = T + I, an error E of P reaches P' as
+// T^T E T, which keeps its direction: next to a pivot that is nearly singular
+// P' is large along one vector and its error with it, while the other vector's
+// stays small (a bound by norms alone proved 67 % instead of 89 % of the counts
+// at random velocities of the uniform batch). The computed element differs
+// from the exact one in three ways:
 //  * its common denominator (relative error th: the sum of the magnitudes of
 //    D's terms over |D|) scales K11, K12, K22 together, which changes the
-//    element's energy, at most 2 q1 + 2 (q1 + q2) ||R|| + ||K11|| ||R||^2 with
+//    element's energy, at most 2 q1 + 2 (q1 + q2) R + R^T K11 R with
 //    q1 = max(|A + E|, |D + G|), q2 = |B| + |F|, by th;
 //  * its numerators (the sums of the magnitudes of their terms over |D|): an
-//    error dn of K11 enters as dn ||R||^2, dd of A + E and D + G as
-//    2 dd (1 + ||R||), dO of B and F as 2 dO ||R||;
+//    error dn of K11 enters as dn R^T R, dd of A + E and D + G as
+//    2 dd (1 + R), dO of B and F as 2 dO R (2 x R <= x (I + R^T R));
 //  * the rounded inputs (k, h, c, moduli), in effect another layer within a
-//    few eps: the kinetic energy's rho c^2 min(kh, 1) (1 + ||T||^2), and,
+//    few eps: the kinetic energy's kin = rho c^2 min(kh, 1) (I + T^T T), and,
 //    for the phases x = k h |w|, whose error grows with k h q / |w| (an
-//    error of q moves w^2 = 1 - q by as much), a factor `amp` on the others.
-// The Schur step's own rounding adds eps (||W|| ||R|| cond(S) + ||P|| + 2 q1).
+//    error of q moves w^2 = 1 - q by as much), a factor `amp` on all of these.
+// The Schur step's own rounding adds eps (||X|| ||S^-1 X|| cond(S) + ||Q||) for
+// P' = Q - X^T S^-1 X. Every S + error is nonsingular when the eigenvalues of
+// E^(1/2) S^-1 E^(1/2) stay below 1 in magnitude; 1/2 is asked.
 // The constants in front of eps were set by measuring the error of P against
-// the double-float recurrence, layer by layer: the largest error was 0.25 of
-// the bound over 1.9 million evaluations of the uniform and ragged workloads
-// (around the root and at random velocities) and 0.65 of it over 0.39 million
-// of models far outside them (thicknesses 0.05..50 m at wavelengths
-// 0.5..500 m); the pivots' condition (error below half the smallest
-// eigenvalue) has a further factor of two in hand. No proven count differed
-// from the double-float one. The bound proves both counts of 90 % (uniform)
-// and 82 % (ragged) of the items and one of the two for nearly all others.
-// (With the plain P' = K22 - K21 S^-1 K12 and its larger bound it was 68 and
-// 65 %, and the count itself was wrong at 10 times as many points.)
+// the double-float recurrence, layer by layer: the largest eigenvalue of
+// E^-1 error was 0.35 over 1.9 million evaluations of the uniform and
+// ragged workloads (around the root and at random velocities) and 0.64
+// over 0.39 million of models far outside them (thicknesses 0.05..50 m at
+// wavelengths 0.5..500 m). No proven count differed
+// from the double-float one. The bound proves both counts of 95 % (uniform)
+// and 92 % (ragged) of the items and one of the two for nearly all others.
 //
 // The element is the screen's (masw_screen.cuh), with 1 - E_r E_s from the
 // e^-x - 1 it is made of.
@@ -161,8 +164,8 @@ static __device__ __noinline__ ElemBound elem_bound_trig(float kh, float pp, flo
     return o;
 }
 
-// The state of the recurrence: P and the bound e of its error's 2-norm.
-struct BoundState { float p00, p01, p11, e; };
+// The state of the recurrence: P and the bound E of its error, -E <= error <= E.
+struct BoundState { float p00, p01, p11, e00, e01, e11; };
 
 // Eliminates one layer's top node: the number of negative eigenvalues of its
 // pivot; *sure is cleared when the pivot's inertia is not proven. BOUND false:
@@ -216,39 +219,53 @@ __device__ __forceinline__ int bound_layer(BoundState& st, const float* __restri
     const float s00 = st.p00 + n00, s01 = st.p01 + n01, s11 = st.p11 + n11;
     const float det = fmaf(s00, s11, -s01 * s01);
     const float idet = rcp_approx(det);
-    // W = P + K11 + K12, R = S^-1 W, P' = P + 2 diag(A + E, D + G) - W^T R
-    const float w00 = st.p00 + aE, w11 = st.p11 + dG, w01 = s01 + cf, w10 = s01 - cf;
-    const float t00 = idet * fmaf(s11, w00, -s01 * w10), t01 = idet * fmaf(s11, w01, -s01 * w11);
-    const float t10 = idet * fmaf(s00, w10, -s01 * w00), t11 = idet * fmaf(s00, w11, -s01 * w01);
     const float ai = fabsf(idet), afr = fabsf(fr);
-    const float mS = norm_2x2(s00, s01, s11), cond = mS * mS * ai;
-    const float q1 = fmaxf(fabsf(aE), fabsf(dG)), q2 = fabsf(n01) + fabsf(cf);
-    const float pn = norm_2x2(st.p00, st.p01, st.p11);
-    st.p00 = fmaf(2.0f, aE, st.p00) - fmaf(w00, t00, w10 * t10);
-    st.p01 = st.p01 - fmaf(w00, t01, w10 * t11);
-    st.p11 = fmaf(2.0f, dG, st.p11) - fmaf(w01, t01, w11 * t11);
+    // P' = Q - X^T Y, Y = S^-1 X: X = W = P + K11 + K12, Q = P + 2 diag(A + E, D + G)
+    // for a thin layer, X = K12, Q = K22 for a thick one, whichever X is smaller
+    const float ce = aE - n00, cg = dG - n11;
+    const float q1 = fmaxf(fabsf(aE), fabsf(dG)), pn = norm_2x2(st.p00, st.p01, st.p11);
+    const float q2 = fabsf(n01) + fabsf(cf);
+    const float mW = pn + q1 + q2, m12 = norm_2x2(ce, cf, cg);
+    const bool thin = mW < m12;
+    const float w00 = thin ? st.p00 + aE : ce, w11 = thin ? st.p11 + dG : cg;
+    const float w01 = thin ? s01 + cf : cf, w10 = thin ? s01 - cf : -cf;
+    const float y00 = idet * fmaf(s11, w00, -s01 * w10), y01 = idet * fmaf(s11, w01, -s01 * w11);
+    const float y10 = idet * fmaf(s00, w10, -s01 * w00), y11 = idet * fmaf(s00, w11, -s01 * w01);
+    st.p00 = (thin ? fmaf(2.0f, aE, st.p00) : n00) - fmaf(w00, y00, w10 * y10);
+    st.p01 = (thin ? st.p01 : -n01) - fmaf(w00, y01, w10 * y11);
+    st.p11 = (thin ? fmaf(2.0f, dG, st.p11) : n11) - fmaf(w01, y01, w11 * y11);
     if (!BOUND) return neg_eigs_2x2(det, s00);
     // the bound
     const float M = norm_2x2(n00, n01, n11);
     const float dO = o.ca * fmaf(fabsf(fm), o.tB, afr * o.tF);
     const float dn = fmaf(o.ca * afr, o.t1, dO), dd = o.ca * afr * o.t2;
     const float th = o.ca * fmaf(o.tD, fabsf(iD), 1.0f);
-    const float eS = st.e + fmaf(th, M, dn) + BOUND_EPS * mS;
-    const float rho = eS * mS * ai;  // >= ||error of S|| ||S^-1||
+    const float mS = norm_2x2(s00, s01, s11), cond = mS * mS * ai;
+    const float loc = fmaf(th, M, fmaf(BOUND_EPS, mS, dn));
+    const float f00 = st.e00 + loc, f11 = st.e11 + loc;
+    // the largest eigenvalue of E^(1/2) S^-1 E^(1/2), at most |trace| + sqrt|det|
+    const float tr = idet * fmaf(s11, f00, fmaf(s00, f11, -2.0f * s01 * st.e01));
+    const float dt = ai * fabsf(fmaf(f00, f11, -st.e01 * st.e01));
+    const float rho = fabsf(tr) + sqrt_approx(dt);
     // (a NaN or infinity anywhere leaves the comparisons false)
     *sure = *sure && (fmaf(4.0f * BOUND_EPS, cond, rho) < 0.5f) && th < BOUND_SCALE;
-    const float R2 = fmaf(t00, t00, t01 * t01) + fmaf(t10, t10, t11 * t11);
-    const float R = sqrt_approx(R2);
-    // T = R - I: its 2-norm from the Frobenius norm and the determinant
-    const float x00 = t00 - 1.0f, x11 = t11 - 1.0f;
-    const float F = fmaf(x00, x00, t01 * t01) + fmaf(x11, x11, t10 * t10);
-    const float dT = fmaf(x00, x11, -t01 * t10);
-    const float T2 = 0.5f * (F + sqrt_approx(fmaxf(fmaf(F, F, -4.0f * dT * dT), 0.0f)));
-    float e = T2 * fmaf(2.0f, rho, 1.0f) * st.e;
-    e = fmaf(th, fmaf(2.0f * R, q1 + q2, fmaf(2.0f, q1, M * R2)), e);
-    e = fmaf(dn, R2, fmaf(2.0f * dd, 1.0f + R, fmaf(2.0f * dO, R, e)));
-    e = fmaf(BOUND_STEP, fmaf(R * (pn + q1 + q2), cond, fmaf(2.0f, q1, pn)), e);
-    st.e = fmaf(o.ca * fabsf(rc2) * fminf(kh, 1.0f), 1.0f + T2, e);
+    const float kin = o.ca * fabsf(rc2) * fminf(kh, 1.0f);
+    const float cross = fmaf(th, q1 + q2, dd + dO);
+    // R = S^-1 W, T = S^-1 K12 = R - I
+    const float one = thin ? 1.0f : 0.0f;
+    const float x00 = y00 - one, x11 = y11 - one, r00 = x00 + 1.0f, r11 = x11 + 1.0f;
+    const float y2 = fmaxf(fabsf(y00), fabsf(y11)) + fmaxf(fabsf(y01), fabsf(y10));  // >= ||Y||
+    const float mX = thin ? mW : m12, mQ = thin ? fmaf(2.0f, q1, pn) : M;
+    const float al = fmaf(2.0f, fmaf(th, q1, dd), cross) + kin +
+                     fmaf(BOUND_STEP, fmaf(mX * y2, cond, mQ), 4.0f * BOUND_EPS * (st.e00 + st.e11));
+    const float be = fmaf(th, M, dn) + cross;
+    // E' = (1 + 2 rho) T^T (E + kin) T + al + be R^T R
+    const float g = fmaf(2.0f, rho, 1.0f), k00 = st.e00 + kin, k11 = st.e11 + kin, k01 = st.e01;
+    const float v00 = fmaf(k00, x00, k01 * y10), v01 = fmaf(k00, y01, k01 * x11);
+    const float v10 = fmaf(k01, x00, k11 * y10), v11 = fmaf(k01, y01, k11 * x11);
+    st.e00 = fmaf(g, fmaf(x00, v00, y10 * v10), fmaf(be, fmaf(r00, r00, y10 * y10), al));
+    st.e01 = fmaf(g, fmaf(x00, v01, y10 * v11), be * fmaf(r00, y01, y10 * r11));
+    st.e11 = fmaf(g, fmaf(y01, v01, x11 * v11), fmaf(be, fmaf(y01, y01, r11 * r11), al));
     return neg_eigs_2x2(det, s00);
 }
 
@@ -259,7 +276,7 @@ template <bool BOUND = true>
 __device__ __forceinline__ int inertia_bound_f(const float* __restrict__ lay, int N, float k,
                                                float c, bool* sure) {
     const float c2 = c * c;
-    BoundState st{0.0f, 0.0f, 0.0f, 0.0f};
+    BoundState st{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     bool ok = true;
     int cnt = 0;
     for (int j = 0; j < N; ++j) cnt += bound_layer<BOUND>(st, lay + j * LAYER_STRIDE32, k, c2, &ok);
@@ -277,8 +294,11 @@ __device__ __forceinline__ int inertia_bound_f(const float* __restrict__ lay, in
     const float mS = norm_2x2(s00, s01, s11);
     // the half-space block: its terms, and s = sqrt(1 - q), whose error is that of q over s
     const float mH = fmaxf(h00, h11) + LA.y * iden * fmaf(g, q, 2.0f * den) + rc2g * rsqrtf(s2);
-    const float eS = st.e + BOUND_EL * mH + BOUND_EPS * mS;
-    *sure = ok && (fabsf(det) > mS * fmaf(4.0f * BOUND_EPS, mS, 2.0f * eS));
+    const float loc = BOUND_EL * mH + BOUND_EPS * mS;
+    const float f00 = st.e00 + loc, f11 = st.e11 + loc, idet = rcp_approx(det);
+    const float tr = idet * fmaf(s11, f00, fmaf(s00, f11, -2.0f * s01 * st.e01));
+    const float dt = fabsf(idet * fmaf(f00, f11, -st.e01 * st.e01));
+    *sure = ok && (fmaf(4.0f * BOUND_EPS * mS * mS, fabsf(idet), fabsf(tr) + sqrt_approx(dt)) < 0.5f);
     return cnt + neg_eigs_2x2(det, s00);
 }
 
