@@ -107,7 +107,7 @@ struct masw_batch {
     int32_t* d_chg_idx = nullptr;
     int32_t* d_chg_status = nullptr;
     int32_t* d_chg_delta = nullptr;
-    int32_t* d_chg_counters = nullptr;  // CHANGES_COUNTERS, then an n_items list
+    int32_t* d_chg_counters = nullptr;  // CHANGES_COUNTERS, then CHANGES_WORK_INTS per item
     bool changes_counted = false;
     // leaky continuation (allocated on first use): per-item outputs, counter
     double* d_lk_ct = nullptr;
@@ -805,7 +805,7 @@ int masw_dispersion_changes(masw_batch* B, int32_t max_changes, double* ct, int3
             return MASW_ENOMEM;
         B->chg_cap = max_changes;
     }
-    if (!B->d_chg_counters && dev_alloc(&B->d_chg_counters, CHANGES_COUNTERS + nw))
+    if (!B->d_chg_counters && dev_alloc(&B->d_chg_counters, CHANGES_COUNTERS + CHANGES_WORK_INTS * nw))
         return MASW_ENOMEM;
     // the first change: Algorithm 1 with the batch plan (an FP64 decision)
     int rc0 = run_scan(B);

@@ -302,4 +302,65 @@ __device__ __forceinline__ int inertia_bound_f(const float* __restrict__ lay, in
     return cnt + neg_eigs_2x2(det, s00);
 }
 
+// clamped_modes_f (masw_screen.cuh) with *sure cleared when one of the signs it
+// rests on is not proven: a numerator or denominator within its error, the
+// element's constant times the amplitudes of its terms, the phase's part (amp
+// at that level's thickness) and the doublings' (2 per level) included, and a
+// further factor of four. The level is taken from a slightly larger x: any
+// level whose pieces lie under the pole-free bound gives the count.
+__device__ __forceinline__ int clamped_modes_bound_f(const float* __restrict__ L, float k, float c2,
+                                                     bool* sure) {
+    const float q = c2 * L[F_IB2];
+    if (!(q > 1.0f - 1.0e-5f)) return 0;
+    const float kh = k * L[F_H], q1 = fmaxf(q - 1.0f, 0.0f);
+    const float x = 1.001f * fmaf(kh, sqrtf(q1) * 0.318309886f, 1.0e-3f);  // kh sqrt(q - 1) / pi
+    if (!(x >= 1.0f)) return 0;
+    if (!(x < 1.0e30f)) {
+        *sure = false;
+        return 0;
+    }
+    const int lv = ((__float_as_int(x) >> 23) & 0xff) - 126;  // 2^lv > x >= 2^(lv-1)
+    float khj = kh * __int_as_float((127 - lv) << 23);        // kh 2^-lv, exact
+    const float r2 = fmaf(-c2, L[F_IA2], 1.0f), s2 = 1.0f - q;
+    WaveF R = wave_fns_f(khj, r2), S = wave_fns_f(khj, s2);
+    const float ar = fmaxf(sqrt_approx(fabsf(r2)), 1.0e-3f), as = fmaxf(sqrt_approx(fabsf(s2)), 1.0e-3f);
+    const float ir = rcp_approx(ar), is = rcp_approx(as);
+    float grow = 1.0f;
+    int J = 0;
+    for (int j = lv; j >= 1; --j) {
+        if (j < lv) {
+            R = WaveF{R.E * R.E, fmaf(2.0f * R.C, R.C, -R.E * R.E), 2.0f * R.Sd * R.C,
+                      2.0f * R.Sm * R.C};
+            S = WaveF{S.E * S.E, fmaf(2.0f * S.C, S.C, -S.E * S.E), 2.0f * S.Sd * S.C,
+                      2.0f * S.Sm * S.C};
+            khj *= 2.0f;
+            grow *= 2.0f;
+        }
+        const float D = fmaf(2.0f, fmaf(R.E, S.E, -R.C * S.C), fmaf(R.Sd, S.Sd, R.Sm * S.Sm));
+        const float an = fmaf(R.C, S.Sd, -S.C * R.Sm);
+        const float dn = fmaf(S.C, R.Sd, -R.C * S.Sm);
+        const float amp = 0.5f * khj * (q * fminf(khj, is) + c2 * L[F_IA2] * fminf(khj, ir));
+        const float tol = 4.0f * BOUND_EL * (grow + amp);
+        // amplitudes: C <= 1, Sd <= min(1/w, kh), Sm <= w (each times at most 1)
+        const float mr = fminf(ir, khj), ms = fminf(is, khj);
+        if (!(fabsf(D) > tol * fmaf(mr, ms, fmaf(ar, as, 4.0f)) && fabsf(an) > tol * (ms + ar) &&
+              fabsf(dn) > tol * (mr + as)))
+            *sure = false;
+        J = 2 * J + (int)((an < 0.0f) != (D < 0.0f)) + (int)((dn < 0.0f) != (D < 0.0f));
+    }
+    return J;
+}
+
+// The mode count T = s + 2 J0 with its proof (inertia_bound_f,
+// clamped_modes_bound_f).
+__device__ __forceinline__ int mode_count_bound_f(const float* __restrict__ lay, int N, float k,
+                                                  float c, int* s_out, bool* sure) {
+    const int s = inertia_bound_f(lay, N, k, c, sure);
+    const float c2 = c * c;
+    int j0 = 0;
+    for (int j = 0; j < N; ++j) j0 += clamped_modes_bound_f(lay + j * LAYER_STRIDE32, k, c2, sure);
+    *s_out = s;
+    return s + 2 * j0;
+}
+
 }  // namespace masw

@@ -112,10 +112,12 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
 // negative-eigenvalue count changes, from the first change `first` (the batch
 // scan's index, -1: none); outputs [n_items][M]. counting 0: FP64 linear scan
 // from one point below it; 1: FP64 search on the monotone mode count
-// s + 2 J0, items whose counts fail going to the linear scan (linear:
-// n_items entries). counters: CHANGES_COUNTERS, [1] = linear-scan items
-// (masw_kernels.cu).
-constexpr int CHANGES_COUNTERS = 2;
+// s + 2 J0, items whose counts fail going to the linear scan. counters:
+// CHANGES_COUNTERS, [1] = linear-scan items, [2] and [3] items the rounds
+// hand on, [4..] open points per round; linear: CHANGES_WORK_INTS per item (the list of
+// linear-scan items, then the rounds' state and lists) (masw_kernels.cu).
+constexpr int CHANGES_COUNTERS = 24;
+constexpr int CHANGES_WORK_INTS = 1 + 8 + 2 + 2;
 cudaError_t launch_changes(const DevBatch& b, const ScanPlan& p, int M, const int32_t* first,
                            const int32_t* cert_counts, const float* layers32, double* ct, int32_t* idx, int32_t* status,
                            int32_t* delta, int32_t* counters, int32_t* linear, int counting,

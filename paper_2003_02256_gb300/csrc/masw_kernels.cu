@@ -33,7 +33,10 @@
 //                         rises).
 //  resolve64_kernel       items whose FP64 counts failed: FP64 scan from V[0].
 // Beyond the first change:
-//  changes_count64_kernel higher modes, FP32 search on the mode count, each
+//  changes_round_kernel,  higher modes, FP32 search on the mode count with its
+//  changes_open_kernel,   error bound, the open points on the FP64 count, the
+//  changes_rest_kernel    few items left after the rounds by a warp each;
+//  changes_count64_kernel the others: FP32 search on the mode count, each
 //                         event certified on the FP64 count;
 //  changes_scan64_kernel  higher modes, FP64 scan at every grid point.
 //  leaky_scan64_kernel    the whole grid with the sign of Re det K (complex
@@ -1260,7 +1263,228 @@ __global__ void __launch_bounds__(256) changes_scan64_kernel(DevBatch b, Changes
     }
 }
 
-// Counting form (plan precision >= 1): a pair of lanes per item checks the
+// Counting form (plan precision >= 1), in rounds over all items: from its last
+// event P an item searches the first point n whose FP32 mode count exceeds T(P)
+// and takes T at n and n - 1 with the FP32 error bound (mode_count_bound_f);
+// the points that the bound leaves open, an eighth of them, go to a list and
+// take the FP64 count (changes_open_kernel), a thread each: in the items' own
+// threads nearly every warp would hold one and run the FP64 code for it. The
+// next round reads the counts: T(V[n-1]) = T(P) and T(V[n]) > T(P) make n the
+// next event, a change when the jump is odd. Items still running after M + 1
+// rounds (an even jump, the FP32 count off by a point next to an event) go to
+// changes_rest_kernel; those whose first change was not certified in the
+// pole-free range, whose FP64 counts fail, or under test routing to
+// changes_count64_kernel.
+// G lanes per item (1, or 4 for batches that would leave the GPU idle). Bound
+// by FP32 instruction issue; with every count in FP64 in one kernel the
+// higher modes of the uniform batch (3 changes) took 2.36 ms, here 1.45.
+struct ChangesState {   // per item
+    int32_t n, T, s;    // the last event P
+    int32_t cand;       // the point in question: n, or 0 (finished), -1 (handed on)
+    int32_t found;      // changes written
+    int32_t Ta, Tc, sc; // T at cand - 1, T and s at cand
+};
+struct ChangesWork {
+    ChangesState* st;   // [n_items]
+    int32_t* open;      // points left to the FP64 count: 2 item + (0: cand - 1, 1: cand)
+    int32_t* n_open;    // [rounds]
+    int32_t* rest;      // items for changes_rest_kernel
+    int32_t* n_rest;
+    int32_t* hard;      // items for changes_count64_kernel
+    int32_t* n_hard;
+};
+// round 0 starts the items, round `last` only reads counts.
+template <int G>
+__global__ void __launch_bounds__(128) changes_round_kernel(
+    DevBatch b, ChangesOut o, int M, int round, int last, const int32_t* __restrict__ first,
+    const int32_t* __restrict__ cert_counts, const float* __restrict__ layers32, ChangesWork w) {
+    const int item = (blockIdx.x * 128 + threadIdx.x) / G;
+    if (item >= b.n_items) return;  // a group's lanes leave together
+    const int gl = threadIdx.x & (G - 1), g0 = (threadIdx.x & 31) - gl;
+    const unsigned gmask = G == 32 ? FULL : ((1u << G) - 1u) << g0;
+    const size_t e0 = (size_t)item * M;
+    const int m = b.item_model[item];
+    const int top = b.model_nlim[m] - 1;
+    ChangesState st;
+    bool rest = false;
+    if (round == 0) {
+        const int n1 = first[item], cc = cert_counts ? cert_counts[item] : -1;
+        const int d = (cc >> 16) - (cc & 0xffff);
+        st = ChangesState{n1, cc >> 16, cc >> 16, 1, 0, 0, 0, 0};
+        if (n1 < 1) st.cand = 0;
+        else if (cc < 0 || b.route != 0 || !(d & 1)) st.cand = -1;
+        else {  // the certificate's counts (J0 = 0 there)
+            if (gl == 0) write_change(b, o, e0, n1, d);
+            st.found = 1;
+        }
+    } else {
+        st = w.st[item];
+        if (st.cand <= 0) return;
+        const int n = st.cand;
+        if (st.Ta < 0 || st.Tc < 0 || st.Ta < st.T || st.Tc < st.Ta) {
+            st.cand = -1;  // the FP64 counts fail
+        } else if (st.Ta == st.T && st.Tc > st.T) {
+            if ((st.Tc - st.T) & 1) {
+                if (gl == 0) write_change(b, o, e0 + st.found, n, st.sc - st.s);
+                ++st.found;
+            }
+            st.n = n;
+            st.T = st.Tc;
+            st.s = st.sc;
+        } else if (st.Tc == st.T && n == top) {
+            st.cand = 0;  // no event up to the limit
+        } else {
+            rest = true;
+        }
+    }
+    if (st.cand > 0 && (st.found >= M || st.n >= top)) st.cand = 0;
+    rest = st.cand > 0 && (rest || round == last);
+    if (rest || st.cand <= 0) {
+        if (gl) return;
+        if (rest) {
+            w.st[item] = st;
+            w.rest[atomicAdd(w.n_rest, 1)] = item;
+        } else if (st.cand < 0) {
+            w.hard[atomicAdd(w.n_hard, 1)] = item;
+        } else {
+            for (int mi = st.found; mi < M; ++mi) write_change(b, o, e0 + mi, -1, 0);
+        }
+        w.st[item].cand = 0;
+        return;
+    }
+    const int l0 = b.model_loff[m];
+    const int N = b.model_loff[m + 1] - l0 - 1;
+    const float* lay32 = layers32 + (size_t)l0 * LAYER_STRIDE32;
+    const float kf = (float)b.k[item];
+    int lo = st.n, hi = top;
+    while (hi - lo > 1) {
+        const int p = section_point<G>(lo, hi, gl);
+        const int c = p < hi ? mode_count_T_f(lay32, N, kf, (float)grid_c(b.c0, b.dc, p)) : st.T + 1;
+        const unsigned mk = (__ballot_sync(gmask, c > st.T) >> g0) & (G == 32 ? ~0u : (1u << G) - 1u);
+        const int f = mk ? __ffs(mk) - 1 : G;
+        const int up = __shfl_sync(gmask, p, g0 + min(f, G - 1));
+        const int dn = __shfl_sync(gmask, p, g0 + max(f - 1, 0));
+        if (f < G) hi = up;
+        if (f > 0) lo = dn;
+    }
+    st.cand = hi;
+    ChangesState* const out = w.st + item;
+    for (int q = gl; q < 2; q += G) {
+        const int pt = hi - 1 + q;
+        int T = st.T, sv = st.s;
+        bool sure = true;
+        if (pt > st.n) T = mode_count_bound_f(lay32, N, kf, (float)grid_c(b.c0, b.dc, pt), &sv, &sure);
+        (q ? out->Tc : out->Ta) = T;
+        if (q) out->sc = sv;
+        if (!sure) w.open[atomicAdd(w.n_open + round, 1)] = 2 * item + q;
+    }
+    if (gl == 0) {
+        out->n = st.n;
+        out->T = st.T;
+        out->s = st.s;
+        out->cand = st.cand;
+        out->found = st.found;
+    }
+}
+
+// The open points of a round on the FP64 mode count, a thread each.
+__global__ void __launch_bounds__(128, 4) changes_open_kernel(DevBatch b, ChangesWork w, int round) {
+    const int total = w.n_open[round];
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const int e = w.open[t], item = e >> 1, q = e & 1;
+        const int l0 = b.model_loff[b.item_model[item]];
+        const int N = b.model_loff[b.item_model[item] + 1] - l0 - 1;
+        ChangesState* const st = w.st + item;
+        int sv;
+        const int T = mode_count_T_df(records_df(b, l0), b.layers + (size_t)l0 * LAYER_STRIDE, N,
+                                      b.k[item], grid_c(b.c0, b.dc, st->cand - 1 + q), &sv);
+        (q ? st->Tc : st->Ta) = T;
+        if (q) st->sc = sv;
+    }
+}
+
+// The items that the rounds leave, a warp each: from its last event P the
+// first point n whose FP32 mode count exceeds T(P) (a 32-way split per step),
+// then T at the 32 points around it, with the FP32 bound or, where that leaves
+// it open, in FP64: the first of them above T(P) is the next event. The window
+// moves when the event lies outside it. Short lists (even jumps, misses of the
+// FP32 count): bound by latency, about 100 us an event; a pair of lanes per
+// item took 0.6 ms for a handful of items. An item whose FP64 counts fail
+// goes to the linear scan.
+__global__ void __launch_bounds__(128) changes_rest_kernel(DevBatch b, ChangesOut o, int M,
+                                                           const float* __restrict__ layers32,
+                                                           ChangesWork w, int32_t* linear,
+                                                           int32_t* n_linear) {
+    const int lane = threadIdx.x & 31;
+    const int total = *w.n_rest;
+    const int warps = (gridDim.x * blockDim.x) >> 5;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total; t += warps) {
+        const int item = w.rest[t];
+        const size_t e0 = (size_t)item * M;
+        const int m = b.item_model[item];
+        const int top = b.model_nlim[m] - 1;
+        const int l0 = b.model_loff[m];
+        const int N = b.model_loff[m + 1] - l0 - 1;
+        const float* lay32 = layers32 + (size_t)l0 * LAYER_STRIDE32;
+        const double* lay = b.layers + (size_t)l0 * LAYER_STRIDE;
+        const float* laydf = records_df(b, l0);
+        const double k = b.k[item];
+        const float kf = (float)k;
+        int n = w.st[item].n, T = w.st[item].T, s = w.st[item].s, found = w.st[item].found;
+        bool bad = false;
+        while (found < M && n < top && !bad) {
+            int lo = n, hi = top;
+            while (hi - lo > 1) {
+                const int p = section_point<32>(lo, hi, lane);
+                const int c = p < hi ? mode_count_T_f(lay32, N, kf, (float)grid_c(b.c0, b.dc, p)) : T + 1;
+                const unsigned mk = __ballot_sync(FULL, c > T);
+                const int f = mk ? __ffs(mk) - 1 : 32;
+                const int up = __shfl_sync(FULL, p, min(f, 31)), dn = __shfl_sync(FULL, p, max(f - 1, 0));
+                if (f < 32) hi = up;
+                if (f > 0) lo = dn;
+            }
+            for (int base = max(hi - 16, n + 1);;) {
+                const int pt = base + lane;
+                int Tp = T, sp = s;
+                bool sure = true;
+                if (pt <= top)
+                    Tp = mode_count_bound_f(lay32, N, kf, (float)grid_c(b.c0, b.dc, pt), &sp, &sure);
+                if (!sure) Tp = mode_count_T_df(laydf, lay, N, k, grid_c(b.c0, b.dc, pt), &sp);
+                bad = __any_sync(FULL, Tp < T);  // a failed count, or T not monotone
+                if (bad) break;
+                const unsigned mk = __ballot_sync(FULL, Tp > T);
+                if (!mk) {  // no event up to the window's end
+                    const int end = min(base + 31, top);
+                    s = __shfl_sync(FULL, sp, end - base);
+                    n = end;
+                    break;
+                }
+                const int f = __ffs(mk) - 1;
+                if (f == 0 && base > n + 1) {  // at or below the window's first point
+                    base = max(base - 31, n + 1);
+                    continue;
+                }
+                const int Te = __shfl_sync(FULL, Tp, f), se = __shfl_sync(FULL, sp, f);
+                n = base + f;
+                if ((Te - T) & 1) {
+                    if (lane == 0) write_change(b, o, e0 + found, n, se - s);
+                    ++found;
+                }
+                T = Te;
+                s = se;
+                break;
+            }
+        }
+        if (lane == 0) {
+            if (bad) linear[atomicAdd(n_linear, 1)] = item;
+            else
+                for (int mi = found; mi < M; ++mi) write_change(b, o, e0 + mi, -1, 0);
+        }
+    }
+}
+
+// The items that the rounds hand on (*n_list of them, grid-stride):
+// a pair of lanes per item checks the
 // first change n1 on the mode count (T and s in FP64 at V[n1-1] and V[n1]:
 // T must jump by an odd amount; for items the counting kernel certified inside
 // the pole-free range, cert_counts holds both) and then takes the next M - 1
@@ -1271,53 +1495,55 @@ __global__ void __launch_bounds__(128) changes_count64_kernel(DevBatch b, Change
                                                               const int32_t* __restrict__ first,
                                                               const int32_t* __restrict__ cert_counts,
                                                               const float* __restrict__ layers32,
+                                                              const int32_t* __restrict__ list,
+                                                              const int32_t* __restrict__ n_list,
                                                               int32_t* linear, int32_t* n_linear) {
-    const int t = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 1);
     const int half = threadIdx.x & 1;
     const unsigned pair = 3u << (threadIdx.x & 30);
-    if (t >= b.n_items) return;  // both lanes of a pair leave together
-    // natural item order: a warp's 16 items share a model and have adjacent
-    // wavelengths, so their evaluations take the same branches
-    const int item = t;
-    const size_t e0 = (size_t)item * M;
-    const int n1 = first[item];
-    int found = 0;
-    bool bad = false;
-    if (n1 >= 1) {
-        const int m = b.item_model[item];
-        const int l0 = b.model_loff[m];
-        const int N = b.model_loff[m + 1] - l0 - 1;
-        const double* lay = b.layers + (size_t)l0 * LAYER_STRIDE;
-        const double k = b.k[item];
-        TPoint below, P;
-        const float* laydf = records_df(b, l0);
-        const int cc = cert_counts ? cert_counts[item] : -1;
-        if (cc >= 0) {  // the certificate's FP64 counts (J0 = 0 there)
-            below = TPoint{n1 - 1, cc & 0xffff, cc & 0xffff};
-            P = TPoint{n1, cc >> 16, cc >> 16};
-        } else {
-            eval_pair(laydf, lay, N, k, b.c0, b.dc, n1 - 1, n1, half, pair, &below, &P);
+    const int total = *n_list;
+    const int stride = (gridDim.x * blockDim.x) >> 1;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 1; t < total; t += stride) {
+        const int item = list[t];  // both lanes of a pair together
+        const size_t e0 = (size_t)item * M;
+        const int n1 = first[item];
+        int found = 0;
+        bool bad = false;
+        if (n1 >= 1) {
+            const int m = b.item_model[item];
+            const int l0 = b.model_loff[m];
+            const int N = b.model_loff[m + 1] - l0 - 1;
+            const double* lay = b.layers + (size_t)l0 * LAYER_STRIDE;
+            const double k = b.k[item];
+            TPoint below, P;
+            const float* laydf = records_df(b, l0);
+            const int cc = cert_counts ? cert_counts[item] : -1;
+            if (cc >= 0) {  // the certificate's FP64 counts (J0 = 0 there)
+                below = TPoint{n1 - 1, cc & 0xffff, cc & 0xffff};
+                P = TPoint{n1, cc >> 16, cc >> 16};
+            } else {
+                eval_pair(laydf, lay, N, k, b.c0, b.dc, n1 - 1, n1, half, pair, &below, &P);
+            }
+            ModeSearch st = mode_search_init(laydf, lay, N, k, b.c0, b.dc,
+                                             b.model_nlim[m] - 1, half, pair,
+                                             P, TPoint{-1, -1, 0});
+            st.bad = st.bad || below.T < 0 || P.T <= below.T || !((P.T - below.T) & 1);
+            if (half == 0) write_change(b, o, e0, n1, P.s - below.s);
+            found = 1;
+            const float* lay32 = layers32 + (size_t)l0 * LAYER_STRIDE32;
+            st.displace = route_displacement(b.route, item);
+            while (found < M) {
+                int d = 0;
+                const int n = next_change_f32(st, lay32, &d);
+                if (n < 0) break;
+                if (half == 0) write_change(b, o, e0 + found, n, d);
+                ++found;
+            }
+            bad = st.bad || route_level(b.route) >= 3;  // (test routing 3: every item to the linear scan)
+            if (bad && half == 0) linear[atomicAdd(n_linear, 1)] = item;
         }
-        ModeSearch st = mode_search_init(laydf, lay, N, k, b.c0, b.dc,
-                                         b.model_nlim[m] - 1, half, pair,
-                                         P, TPoint{-1, -1, 0});
-        st.bad = st.bad || below.T < 0 || P.T <= below.T || !((P.T - below.T) & 1);
-        if (half == 0) write_change(b, o, e0, n1, P.s - below.s);
-        found = 1;
-        const float* lay32 = layers32 + (size_t)l0 * LAYER_STRIDE32;
-        st.displace = route_displacement(b.route, item);
-        while (found < M) {
-            int d = 0;
-            const int n = next_change_f32(st, lay32, &d);
-            if (n < 0) break;
-            if (half == 0) write_change(b, o, e0 + found, n, d);
-            ++found;
-        }
-        bad = st.bad || route_level(b.route) >= 3;  // (test routing 3: every item to the linear scan)
-        if (bad && half == 0) linear[atomicAdd(n_linear, 1)] = item;
+        if (half == 0 && !bad)
+            for (int mi = found; mi < M; ++mi) write_change(b, o, e0 + mi, -1, 0);
     }
-    if (half == 0 && !bad)
-        for (int mi = found; mi < M; ++mi) write_change(b, o, e0 + mi, -1, 0);
 }
 
 cudaError_t launch_changes(const DevBatch& b, const ScanPlan& p, int M, const int32_t* first,
@@ -1336,9 +1562,37 @@ cudaError_t launch_changes(const DevBatch& b, const ScanPlan& p, int M, const in
                                                           nullptr);
         return cudaGetLastError();
     }
-    const long long threads = 2LL * b.n_items;
-    changes_count64_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(
-        b, o, M, first, cert_counts, layers32, linear, counters + 1);
+    const int sms = p.sms > 0 ? p.sms : 152;
+    ChangesWork w;
+    w.st = reinterpret_cast<ChangesState*>(linear + b.n_items);
+    static_assert(sizeof(ChangesState) == 32, "CHANGES_WORK_INTS counts it");
+    w.open = reinterpret_cast<int32_t*>(w.st + b.n_items);
+    w.rest = w.open + 2 * (size_t)b.n_items;
+    w.hard = w.rest + b.n_items;
+    w.n_hard = counters + 2;
+    w.n_rest = counters + 3;
+    w.n_open = counters + 4;
+    int32_t* const hard = w.hard;
+    const int rounds = M + 1;  // an event per round, and two even jumps
+    const bool groups = b.n_items < 65536;  // (4 lanes per item fill the GPU up to there)
+    for (int r = 0; r <= rounds; ++r) {
+        if (groups)
+            changes_round_kernel<4><<<(unsigned)((4LL * b.n_items + 127) / 128), 128, 0, s>>>(
+                b, o, M, r, rounds, first, cert_counts, layers32, w);
+        else
+            changes_round_kernel<1><<<(b.n_items + 127) / 128, 128, 0, s>>>(
+                b, o, M, r, rounds, first, cert_counts, layers32, w);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (r == rounds) break;
+        changes_open_kernel<<<std::max(1, std::min(4 * sms, (2 * b.n_items + 127) / 128)), 128, 0, s>>>(
+            b, w, r);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    changes_rest_kernel<<<std::max(1, std::min(4 * sms, (b.n_items + 3) / 4)), 128, 0, s>>>(
+        b, o, M, layers32, w, linear, counters + 1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    changes_count64_kernel<<<std::max(1, std::min(4 * sms, (b.n_items + 63) / 64)), 128, 0, s>>>(
+        b, o, M, first, cert_counts, layers32, hard, counters + 2, linear, counters + 1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     changes_scan64_kernel<<<lblocks, 32 * wpb, 0, s>>>(b, o, M, first, counters, linear,

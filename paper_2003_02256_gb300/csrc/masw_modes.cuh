@@ -23,6 +23,7 @@
 // certifies it on the FP64 count, with next_change as its fallback.
 #pragma once
 
+#include "masw_bound.cuh"
 #include "masw_device.cuh"
 #include "masw_df.cuh"
 #include "masw_screen.cuh"
