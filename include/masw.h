@@ -112,11 +112,11 @@ typedef struct {
                                 else decided on the FP64 count; items
                                 outside the bound take the linear screen of 1. Default: 2 */
     int32_t count_block;     /* precision 2: threads per block of the counting kernel, 64, 128
-                                or 256 (two lanes per item, items of a block consecutive;
-                                launch bounds of 14, 7 or 2 resident blocks). Default: 256
-                                with count_split 1 or 2, else 128 */
-    int32_t count_split;     /* precision 2: 0 the search (a lane pair per item, three-way
-                                splits) and the certificate in one kernel; 1 the search
+                                or 256 (items of a block consecutive; launch bounds of
+                                at least 512 resident threads per SM). Default: 256 above
+                                65,536 items, else 128 */
+    int32_t count_split;     /* precision 2: 0 the search (2 to 32 lanes per item by batch
+                                size) and the certificate in one kernel; 1 the search
                                 in kernels of their own (one thread per item: every 6th
                                 wavelength of a model and its last by bisection, then
                                 the others from a guess between those two indices)
@@ -127,7 +127,7 @@ typedef struct {
                                 change below the bound, a mode below V[0]) take that
                                 scan, its check and the mode-count search on a second,
                                 highest-priority stream beside the certificate. Same
-                                results for all three. Default: 0 below 65,536 items,
+                                results for all three. Default: 0 below 98,304 items,
                                 else 2 when the models or the grid as created make
                                 such items likely (a layer slower than the one
                                 above it, a grid above the slowest modes), else 1. With 1 or 2,

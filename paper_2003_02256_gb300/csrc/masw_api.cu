@@ -362,18 +362,18 @@ static masw_plan default_plan(const masw_batch* B) {
     p.stage_layers = std::min(B->max_layers + 1, 32);
     p.use_graph = 1;
     p.precision = 2;
-    // The fused kernel's lane pairs give small batches the shortest chain of
-    // launches; from 65,536 items the split kernels, whose search proves most
-    // certificates, are ahead (32,000 items of 8 layers 125 us fused, 129
-    // split; 64,400 ragged 580 and 584; 80,000 of 8 layers 215 and 171). The
+    // The fused kernel gives small batches the shortest chain of launches;
+    // from 98,304 items the split kernels, whose two passes search with a third
+    // of the evaluations, are ahead (64,000 items of 8 layers 125 us fused, 131
+    // split; 76,800 of 12 layers 190 and 222; 151,600 ragged 1035 and 627). The
     // second stream where the search will leave items to the fallback chain:
     // models with a layer slower than the one above it, or a grid that starts
-    // above a model's slowest modes (701 ragged models 762 -> 630 us with it;
-    // a uniform batch without such items 238 -> 246).
-    p.count_split = B->n_items < (1 << 16) ? 0 : B->fallback_likely ? 2 : 1;
-    // with the split search, blocks of 256 at 2 per SM (128 registers, no
-    // spills) against 128 at 7 (72 registers): uniform batch 257 -> 238 us
-    p.count_block = p.count_split ? 256 : 128;
+    // above a model's slowest modes (701 ragged models 724 -> 627 us with it).
+    p.count_split = B->n_items < 98304 ? 0 : B->fallback_likely ? 2 : 1;
+    // blocks of 256 at 2 per SM (128 registers, no spills) for the split
+    // certificate (uniform batch 257 -> 238 us against 128 at 7) and the
+    // largest fused batches (76,800 items of 12 layers 190 us, 211 with 128)
+    p.count_block = B->n_items > 65536 ? 256 : 128;
     return p;
 }
 

@@ -136,21 +136,26 @@ __device__ __forceinline__ Located count_search_single(const float* __restrict__
         if (inertia_f(lay32, N, kf, fmaf((float)mid, dcf, c0f)) >= 1) hi = mid;
         else lo = mid;
     }
+    // the bounded counts, and where they disagree with the plain ones (thin
+    // layers) a step towards them
 #pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-        const int p = side ? lo : hi;
-        if (p < 0) break;
-        bool sure;
-        const int c = count_bound_at(lay32, N, kf, c0, dc, p, &sure);
-        if (side) {
-            if (sure && c == 0) r.proof |= PROOF_LO;
-        } else {
-            if (c < 1 && hi == npf - 1) return r;  // no change inside the range
-            if (sure && (c & 1)) {
-                r.proof |= PROOF_HI;
-                r.count = c;
-            }
+    for (int tries = 0;; ++tries) {
+        bool s_hi, s_lo = false;
+        const int c_hi = count_bound_at(lay32, N, kf, c0, dc, hi, &s_hi);
+        if (c_hi < 1 && hi == npf - 1) return r;  // no change inside the range
+        int c_lo = 0;
+        if (c_hi < 1 && tries < 4) {
+            lo = hi++;
+            continue;
         }
+        if (lo >= 0) c_lo = count_bound_at(lay32, N, kf, c0, dc, lo, &s_lo);
+        if (c_lo >= 1 && tries < 4) {
+            hi = lo--;
+            continue;
+        }
+        r.proof = (s_lo && c_lo == 0 ? PROOF_LO : 0) | (s_hi && (c_hi & 1) ? PROOF_HI : 0);
+        r.count = c_hi;
+        break;
     }
     r.n = hi;
     return r;
@@ -237,28 +242,37 @@ __device__ __forceinline__ Located count_search_group(const float* __restrict__ 
                                                       int gl, int g0, unsigned gmask) {
     Located r{-1, 0, 0};
     if (npf < 1) return r;
-    const float kf = (float)k;
+    const float kf = (float)k, c0f = (float)c0, dcf = (float)dc;
     int lo = -1, hi = npf - 1;  // (the top is taken as nonzero until the end)
     while (hi - lo > 1) {
         const int p = section_point<G>(lo, hi, gl);
-        const int c = p < hi ? inertia_bound_f<false>(lay32, N, kf, (float)grid_c(c0, dc, p), nullptr) : 1;
+        const int c = p < hi ? inertia_f(lay32, N, kf, fmaf((float)p, dcf, c0f)) : 1;
         const unsigned m = (__ballot_sync(gmask, c >= 1) >> g0) & (G == 32 ? ~0u : (1u << G) - 1u);
         const int f = m ? __ffs(m) - 1 : G;  // first lane at or above the change
         const int top = __shfl_sync(gmask, p, g0 + min(f, G - 1)), below = __shfl_sync(gmask, p, g0 + max(f - 1, 0));
         if (f < G) hi = top;
         if (f > 0) lo = below;
     }
-    // even lanes V[lo], odd lanes V[hi]
-    const int p = (gl & 1) ? hi : lo;
-    bool sure = false;
-    const int c = p >= 0 ? count_bound_at(lay32, N, kf, c0, dc, p, &sure) : 0;
-    const int c_lo = __shfl_sync(gmask, c, g0), c_hi = __shfl_sync(gmask, c, g0 + 1);
-    const bool s_lo = __shfl_sync(gmask, (int)sure, g0), s_hi = __shfl_sync(gmask, (int)sure, g0 + 1);
-    if (c_hi < 1 && hi == npf - 1) return r;  // no change inside the range
-    r.n = hi;
-    r.proof = (s_lo && c_lo == 0 ? PROOF_LO : 0) | (s_hi && (c_hi & 1) ? PROOF_HI : 0);
-    r.count = c_hi;
-    return r;
+    // the bounded counts, even lanes V[lo], odd lanes V[hi], and where they
+    // disagree with the plain ones (thin layers) a step towards them
+    for (int tries = 0;; ++tries) {
+        const int p = (gl & 1) ? hi : lo;
+        bool sure = false;
+        const int c = p >= 0 ? count_bound_at(lay32, N, kf, c0, dc, p, &sure) : 0;
+        const int c_lo = __shfl_sync(gmask, c, g0), c_hi = __shfl_sync(gmask, c, g0 + 1);
+        const bool s_lo = __shfl_sync(gmask, (int)sure, g0), s_hi = __shfl_sync(gmask, (int)sure, g0 + 1);
+        if (c_hi < 1 && hi == npf - 1) return r;  // no change inside the range
+        if (tries < 4 && c_hi < 1) {
+            lo = hi++;
+        } else if (tries < 4 && c_lo >= 1) {
+            hi = lo--;
+        } else {
+            r.n = hi;
+            r.proof = (s_lo && c_lo == 0 ? PROOF_LO : 0) | (s_hi && (c_hi & 1) ? PROOF_HI : 0);
+            r.count = c_hi;
+            return r;
+        }
+    }
 }
 
 // count_search_guess by a group of G lanes: first the points guess - 1 ..
