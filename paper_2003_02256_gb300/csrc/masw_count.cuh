@@ -88,16 +88,6 @@ static __device__ __noinline__ int pair_search(const float* __restrict__ lay32, 
     return hi;
 }
 
-// The search stage: the first grid point in [0, npf) with a nonzero FP32
-// count (count 0 at c = 0: static stiffness positive definite), -1 when
-// there is none or npf < 1. Both lanes get the same index.
-__device__ __forceinline__ int count_search_pair(const float* __restrict__ lay32, int N, double k,
-                                                 double c0, double dc, int npf, int half,
-                                                 unsigned pair) {
-    if (npf < 1) return -1;
-    return pair_search(lay32, N, (float)k, (float)c0, (float)dc, -1, npf - 1, 1, half, pair);
-}
-
 // What the split search knows of an item: its index n (the first grid point
 // in [0, npf) with a nonzero FP32 count, or -1) and which of the counts at
 // V[n-1] and V[n] the FP32 error bound proves (masw_bound.cuh).
@@ -322,7 +312,7 @@ __device__ __forceinline__ Located count_search_guess_group(const float* __restr
     return r;
 }
 
-// The certificate stage for the search's index n (count_search_pair or
+// The certificate stage for the search's index n (count_search_guess or
 // count_search_single) in the
 // pole-free range [0, npf). Both lanes of the pair (lane bit 0 = half, `pair`
 // = their shuffle mask) call it with the same item and get the same result.
@@ -414,18 +404,6 @@ __device__ __forceinline__ PairCount certify_pair(const float* __restrict__ lay3
     out.n = cert >= 1 ? -1 : n;
     if (cert >= 1 && cert < npf) out.counts = pack_counts(s_lo, s_hi);
     return out;
-}
-
-// Search and certificate in one call (count_search_pair, certify_pair).
-// Requires nlim >= 2.
-__device__ __forceinline__ PairCount count_certify_pair(const float* __restrict__ lay32,
-                                                        const float* __restrict__ laydf,
-                                                        const double* __restrict__ lay, int N,
-                                                        double k, double c0, double dc, int nlim,
-                                                        int half, unsigned pair) {
-    const int npf = pole_free_points_f(lay32, N, (float)k, (float)c0, (float)dc, nlim);
-    const int n = count_search_pair(lay32, N, k, c0, dc, npf, half, pair);
-    return certify_pair(lay32, laydf, lay, N, k, c0, dc, nlim, npf, n, half, pair);
 }
 
 }  // namespace masw

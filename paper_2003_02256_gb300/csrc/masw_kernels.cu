@@ -67,13 +67,13 @@
 #include "masw_count.cuh"
 #include "masw_device.cuh"
 #include "masw_df.cuh"
+#include "masw_fused.cuh"
 #include "masw_internal.h"
 #include "masw_modes.cuh"
 #include "masw_screen.cuh"
 
 namespace masw {
 
-constexpr unsigned FULL = 0xffffffffu;
 
 // ------------------------------------------------------------------ scan
 
@@ -698,107 +698,42 @@ __device__ __forceinline__ void certify_item(const DevBatch& b, const float* __r
     }
 }
 
-// One warp, a group of DD_GROUP lanes per item (`on`): items whose counts va at
-// V[n-1] and vb at V[n] are not the certificate's because the FP32 index is off
-// by a point or two. Count 0 at both: the change is higher, the points above
-// in turn; nonzero at V[n-1]: lower, the points below; inside the pole-free
-// range, four points at most, each by det_inertia_dd_group; an even count at
-// V[n]: the first odd one above. Writes the certified
-// result and returns; otherwise lists the item for the sign scan (from the
-// last point known to have an even count, where V[n-1] has count 0). A few
-// items in 100,000: the sign scan after the kernel would cost them, and the
-// whole batch, about 90 us.
-static __device__ __noinline__ void certify_near(const DevBatch& b, const float* __restrict__ layers32,
-                                                 const ScanOut& o, bool on, int item, int n, int va,
-                                                 int vb, float* sh, int32_t* n32, int32_t* search,
-                                                 int32_t* n_search) {
-    const int m = b.item_model[item];
-    const int lo_rec = b.model_loff[m];
-    const int N = b.model_loff[m + 1] - lo_rec - 1;
-    const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
-    const double k = b.k[item];
-    const int npf = on ? pole_free_points_f(layers32 + (size_t)lo_rec * LAYER_STRIDE32, N, (float)k,
-                                            (float)b.c0, (float)b.dc, b.model_nlim[m])
-                       : 0;
-    const bool up = va == 0 && vb == 0, down = va > 0;
-    // the point in hand and its count: 0 going up, nonzero going down
-    int at = up ? n : n - 1, cnt = up ? 0 : va;
-    int cert = -1, s_lo = 0, s_hi = 0;
-    bool go = on && (up || down);
-    for (int tries = 0; tries < 4; ++tries) {
-        const int p = up ? at + 1 : at - 1;
-        go = go && p >= 0 && p < npf;
-        if (!__any_sync(FULL, go)) break;
-        const int v = det_inertia_dd_group(records_df(b, lo_rec), lay, go ? N : 0, k,
-                                           grid_c(b.c0, b.dc, max(p, 0)), sh);
-        if (!go) continue;
-        if (v < 0) {
-            go = false;
-        } else if (up) {
-            if (v > 0) {
-                if (v & 1) {
-                    cert = p;
-                    s_hi = v;
-                }
-                go = false;
-            }
-            if (v == 0 || !(v & 1)) at = p;  // an even count up to here
-        } else if (v == 0) {
-            if (cnt & 1) {
-                cert = at;
-                s_hi = cnt;
-            }
-            go = false;
-        } else {
-            at = p;
-            cnt = v;
-        }
+// The items of a batch for masw_fused.cuh.
+struct BatchSrc {
+    DevBatch b;
+    const float* layers32;
+    ScanOut o;
+    int32_t *n32, *search, *n_search, *fallback_list, *n_fallback;
+    __device__ __forceinline__ double c0() const { return b.c0; }
+    __device__ __forceinline__ double dc() const { return b.dc; }
+    __device__ __forceinline__ int route() const { return route_level(b.route); }
+    __device__ __forceinline__ CountItem get(int item) const {
+        const int m = b.item_model[item], lo = b.model_loff[m];
+        return CountItem{layers32 + (size_t)lo * LAYER_STRIDE32, records_df(b, lo),
+                         b.layers + (size_t)lo * LAYER_STRIDE, b.model_loff[m + 1] - lo - 1,
+                         b.model_nlim[m], b.k[item]};
     }
-    // Two modes inside one interval (count 0, then even): the first odd count
-    // above, located on the FP32 count by the group's lanes, with the even
-    // count one point below it.
-    bool even = on && va == 0 && vb >= 2 && !(vb & 1);
-    if (__any_sync(FULL, even)) {
-        const int gl = threadIdx.x & (DD_GROUP - 1), g0 = (threadIdx.x & 31) - gl;
-        const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
-        int lo = n, hi = npf - 1;
-        even = even && hi > lo;
-        for (;;) {
-            const bool act = even && hi - lo > 1;
-            if (!__any_sync(FULL, act)) break;
-            const int p = act ? section_point<DD_GROUP>(lo, hi, gl) : 0;
-            const int c = act && p < hi
-                              ? inertia_f(lay32, N, (float)k, fmaf((float)p, (float)b.dc, (float)b.c0))
-                              : vb + 1;
-            const unsigned mk = (__ballot_sync(FULL, c > vb) >> g0) & ((1u << DD_GROUP) - 1u);
-            const int f = mk ? __ffs(mk) - 1 : DD_GROUP;
-            const int p_up = __shfl_sync(FULL, p, g0 + min(f, DD_GROUP - 1));
-            const int p_dn = __shfl_sync(FULL, p, g0 + max(f - 1, 0));
-            if (act && f < DD_GROUP) hi = p_up;
-            if (act && f > 0) lo = p_dn;
-        }
-        const int ua = det_inertia_dd_group(records_df(b, lo_rec), lay, even && hi - 1 > n ? N : 0, k,
-                                            grid_c(b.c0, b.dc, max(hi - 1, 0)), sh);
-        const int ub = det_inertia_dd_group(records_df(b, lo_rec), lay, even ? N : 0, k,
-                                            grid_c(b.c0, b.dc, max(hi, 0)), sh);
-        if (even && (hi - 1 == n || ua == vb) && ub > vb && (ub & 1)) {
-            cert = hi;
-            s_lo = vb;
-            s_hi = ub;
-        }
-    }
-    if (!on || (threadIdx.x & (DD_GROUP - 1))) return;
-    if (cert >= 1) {
-        n32[item] = cert | SCREEN_COUNTED;
-        write_result(b, o, item, cert);
-        if (o.cert_counts) o.cert_counts[item] = pack_counts(s_lo, s_hi);
-    } else {
-        // with an even count at V[n], or going up, to `at`, else to V[n-1]
-        n32[item] = up ? at : (vb >= 0 && !(vb & 1)) ? n : n - 1;
+    __device__ __forceinline__ void none(int item) const {
+        n32[item] = -1;
+        write_result(b, o, item, -1);
         if (o.cert_counts) o.cert_counts[item] = -1;
-        search[atomicAdd(n_search, 1)] = item | (va == 0 ? SCAN_FROM : 0);
     }
-}
+    __device__ __forceinline__ void fallback(int item, int start) const {
+        n32[item] = start;
+        if (o.cert_counts) o.cert_counts[item] = -1;
+        fallback_list[atomicAdd(n_fallback, 1)] = item;
+    }
+    __device__ __forceinline__ void done(int item, int n, int s_lo, int s_hi) const {
+        n32[item] = n | SCREEN_COUNTED;
+        write_result(b, o, item, n);
+        if (o.cert_counts) o.cert_counts[item] = pack_counts(s_lo, s_hi);
+    }
+    __device__ __forceinline__ void missed(int item, int n, bool from) const {
+        n32[item] = n;
+        if (o.cert_counts) o.cert_counts[item] = -1;
+        search[atomicAdd(n_search, 1)] = item | (from ? SCAN_FROM : 0);
+    }
+};
 
 // The split search's lists (device-side counts, grid-stride). The
 // items of w.two (neither count proven) take a pair of lanes each; those of
@@ -844,8 +779,8 @@ __global__ void __launch_bounds__(B, (B == 256 ? 2 : B == 64 ? 10 : 7))
                 if (o.cert_counts) o.cert_counts[it] = pack_counts(0, vb);
             }
             if (__any_sync(FULL, mine && !ok))
-                certify_near(b, layers32, o, mine && !ok, it, n, low ? v : 0, vb,
-                             s_dd[threadIdx.x / DD_GROUP], w.n32, search, n_search);
+                certify_near(BatchSrc{b, layers32, o, w.n32, search, n_search, fallback, n_fallback},
+                             mine && !ok, it, n, low ? v : 0, vb, s_dd[threadIdx.x / DD_GROUP]);
         }
     }
     for (int t = (blockIdx.x * B + threadIdx.x) >> 1; t < end; t += stride) {
@@ -887,108 +822,11 @@ __global__ void __launch_bounds__(B, (B == 256 ? 2 : B == 64 ? 10 : 7))
     }
 }
 
-// The fused plan (count_split 0, smaller batches): G lanes per item search
-// it (count_search_group) with the FP32 bound's proofs; the points that the
-// bound leaves open, a twentieth of them, are collected in shared memory and
-// take the double-float count, 8 lanes of the block each
-// (det_inertia_dd_group): in the items' own lanes
-// nearly every warp would hold one and run the double-float code for it. An
-// item whose counts are not the certificate's takes certify_near; items the search
-// cannot place go to the fallback list. Bound by latency: G splits the range in
-// G + 1 per step. (A lane pair per item with a double-float count on each
-// lane: one curve of 60 items 45 us, here 20; 9,600 items of 8 layers 94, here
-// 57; 64,000 of 8 layers 175, here 125; 76,800 of 12 layers 300, here 190.)
-// Launch bounds: 768 threads per SM for pairs (85 registers, 64,000 items 125
-// us against 140 at 512), 512 for the wider groups, whose latency counts.
+// The fused plan (count_split 0, smaller batches), masw_fused.cuh.
 template <int B, int G>
 __global__ void __launch_bounds__(B, (B == 256 ? 2 : (G == 2 ? 768 : 512) / B))
-    count_fused_kernel(DevBatch b, const float* __restrict__ layers32, ScanOut o, int32_t* n32,
-                       int32_t* search, int32_t* n_search, int32_t* fallback, int32_t* n_fallback,
-                       int item_begin, int item_end) {
-    constexpr int ITEMS = B / G;
-    __shared__ int s_n, s_open[2 * ITEMS], s_at[2 * ITEMS], s_count[2 * ITEMS];
-    __shared__ __align__(8) float s_dd[B / DD_GROUP][DD_GROUP_FLOATS];
-    const int tid = threadIdx.x;
-    const int slot = tid / G, gl = tid & (G - 1), g0 = (tid & 31) - gl;
-    const unsigned gmask = G == 32 ? FULL : ((1u << G) - 1u) << g0;
-    const int item0 = item_begin + blockIdx.x * ITEMS;
-    const int item = item0 + slot;
-    if (tid == 0) s_n = 0;
-    __syncthreads();
-    Located r{-1, 0, 0};
-    bool open = false;  // leader lane: counts still wanted
-    if (item < item_end) {
-        const int m = b.item_model[item];
-        const int lo_rec = b.model_loff[m];
-        const int N = b.model_loff[m + 1] - lo_rec - 1;
-        const int nlim = b.model_nlim[m];
-        const float* lay32 = layers32 + (size_t)lo_rec * LAYER_STRIDE32;
-        const double k = b.k[item];
-        int npf = 0;
-        if (nlim >= 2) {
-            npf = pole_free_points_f(lay32, N, (float)k, (float)b.c0, (float)b.dc, nlim);
-            r = count_search_group<G>(lay32, N, k, b.c0, b.dc, npf, gl, g0, gmask);
-        }
-        if (gl == 0) {
-            if (nlim < 2) {
-                n32[item] = -1;
-                write_result(b, o, item, -1);
-                if (o.cert_counts) o.cert_counts[item] = -1;
-            } else if (r.n < 1 || route_level(b.route) >= 1) {
-                // the start of the linear FP32 scan: the end of the range when
-                // it holds no change, else (test routing too) V[0]
-                n32[item] = (route_level(b.route) < 1 && npf >= 1 && r.n < 0) ? npf : 0;
-                if (o.cert_counts) o.cert_counts[item] = -1;
-                fallback[atomicAdd(n_fallback, 1)] = item;
-            } else {
-                open = true;
-                s_count[2 * slot] = 0;
-                s_count[2 * slot + 1] = r.count;
-                for (int side = 0; side < 2; ++side)
-                    if (!(r.proof & (side ? PROOF_HI : PROOF_LO))) {
-                        const int q = atomicAdd(&s_n, 1);
-                        s_open[q] = 2 * slot + side;
-                        s_at[q] = r.n - 1 + side;
-                    }
-            }
-        }
-    }
-    __syncthreads();
-    for (int q0 = 4 * (tid >> 5); q0 < s_n; q0 += B / DD_GROUP) {  // a warp's four groups
-        const int q = q0 + ((tid & 31) / DD_GROUP);
-        const bool mine = q < s_n;
-        const int e = s_open[mine ? q : q0], it = item0 + (e >> 1);
-        const int lo_rec = b.model_loff[b.item_model[it]];
-        const int N = b.model_loff[b.item_model[it] + 1] - lo_rec - 1;
-        const int v = det_inertia_dd_group(records_df(b, lo_rec),
-                                           b.layers + (size_t)lo_rec * LAYER_STRIDE, mine ? N : 0,
-                                           b.k[it], grid_c(b.c0, b.dc, s_at[mine ? q : q0]),
-                                           s_dd[tid / DD_GROUP]);
-        if (mine && (tid & (DD_GROUP - 1)) == 0) s_count[e] = v;
-    }
-    __syncthreads();
-    if (tid == 0) s_n = 0;
-    __syncthreads();
-    if (open) {
-        const int va = s_count[2 * slot], vb = s_count[2 * slot + 1];
-        if (va == 0 && vb > 0 && (vb & 1)) {
-            n32[item] = r.n | SCREEN_COUNTED;
-            write_result(b, o, item, r.n);
-            if (o.cert_counts) o.cert_counts[item] = pack_counts(va, vb);
-        } else {
-            const int q = atomicAdd(&s_n, 1);
-            s_open[q] = slot;
-            s_at[q] = r.n;
-        }
-    }
-    __syncthreads();
-    for (int q0 = 4 * (tid >> 5); q0 < s_n; q0 += B / DD_GROUP) {
-        const int q = q0 + ((tid & 31) / DD_GROUP);
-        const bool mine = q < s_n;
-        const int e = s_open[mine ? q : q0];
-        certify_near(b, layers32, o, mine, item0 + e, s_at[mine ? q : q0], s_count[2 * e],
-                     s_count[2 * e + 1], s_dd[tid / DD_GROUP], n32, search, n_search);
-    }
+    count_fused_kernel(BatchSrc src, int item_begin, int item_end) {
+    count_fused_block<B, G>(src, item_begin, item_end);
 }
 
 // Items that the sign scan hands on (too many points its error bound leaves
@@ -1346,7 +1184,8 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
         const int g = n <= 4096 ? 32 : n <= 16384 ? 8 : n <= 24576 ? 4 : 2;
 #define MASW_FUSED(BS, G)                                                                     \
     count_fused_kernel<BS, G><<<(n + BS / G - 1) / (BS / G), BS, 0, s>>>(                     \
-        b, layers32, o, n32, search, counters + 5, fallback, counters + 3, item_begin, item_end)
+        BatchSrc{b, layers32, o, n32, search, counters + 5, fallback, counters + 3}, item_begin, \
+        item_end)
 #define MASW_COUNT_LAUNCH(BS)                                                                 \
     do {                                                                                      \
         if (p.count_split)                                                                    \

@@ -27,13 +27,11 @@
 //   [FP32 records: rmax x 8 f32] [k: imax f64]
 //   [scan state: imax x (base, carry, phase, located index) i32]
 // Each item runs the default scan of the batch path: in the tick after its
-// admission, a lane pair runs the counting search (the FP32 negative-
-// eigenvalue count split below the pole-free bound) and its FP64 certificate
-// (count 0 at V[n-1], odd at V[n]; count_certify_pair), so most requests
-// finish in one tick; an uncertified item takes the FP64 search on the
-// Wittrick-Williams mode count from V[0] in the same kernel (masw_modes.cuh).
-// Items whose change lies above the bound continue with paired FP32 chunks
-// from the bound, up to `chunks_per_tick` per tick, and get the batch path's
+// admission, a lane group runs the counting search (the FP32 negative-
+// eigenvalue count split below the pole-free bound) and its certificate
+// (count 0 at V[n-1], odd at V[n]; masw_fused.cuh), so most requests
+// finish in one tick. Items whose change lies above the bound, and the few not
+// certified, continue with paired FP32 chunks from the bound, up to `chunks_per_tick` per tick, and get the batch path's
 // three-point FP64 check on the mode count at V[0], V[n-1], V[n]; when it does
 // not confirm, the same mode-count search. Items whose FP64 counts fail
 // continue with FP64 chunks, one per tick, from V[0].
@@ -49,6 +47,7 @@
 #include "../../include/masw.h"
 #include "masw_count.cuh"
 #include "masw_device.cuh"
+#include "masw_fused.cuh"
 #include "masw_internal.h"
 #include "masw_modes.cuh"
 #include "masw_screen.cuh"
@@ -57,7 +56,6 @@ using namespace masw;
 
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
 
 struct SlotView {
     double* region;      // [slots][stride] doubles
@@ -164,52 +162,51 @@ __device__ bool search_or_rescan(SlotView v, int item, int slot, const double* l
     return false;
 }
 
-// Tick, part 0 (two lanes per item admitted since the last tick): the
-// counting search and its FP64 certificate of the batch path
-// (count_certify_pair). A certified item is finished here. When the
-// certificate failed, the pair searches the first change on the FP64 mode
-// count from V[0] (next_change) and finishes the item too (if those counts
-// fail, the FP64 scan from V[0] follows at the next ticks). The fallback
-// items continue at the next tick with the linear FP32 screen from the end of
-// the pole-free range (carrying the positive sign of count 0) or from V[0].
-__global__ void __launch_bounds__(128, 7) serve_count_kernel(SlotView v, const int32_t* __restrict__ items,
-                                                             int n_items, int32_t* active_out,
-                                                             double c0, double dc) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if ((t >> 1) >= n_items) return;  // both lanes of a pair leave together
-    const int half = t & 1;
-    const unsigned pair = 3u << ((threadIdx.x & 31) & 30);
-    const int item = items[t >> 1];
-    const int slot = item / v.imax;
-    const int j = item - slot * v.imax;
-    const int32_t* meta = slot_meta(v, slot);
-    const int N = meta[0] - 1;
-    const int nlim = meta[1];
-    int32_t* stt = slot_state(v, slot) + 4 * j;
-    if (nlim < 2) {
-        if (!half) finish_item(v, item, slot, -1, c0, dc);
-        return;
+// The items admitted since the last tick for masw_fused.cuh.
+struct ServeSrc {
+    SlotView v;
+    const int32_t* items;
+    int32_t* active_out;
+    double c0_, dc_;
+    __device__ __forceinline__ double c0() const { return c0_; }
+    __device__ __forceinline__ double dc() const { return dc_; }
+    __device__ __forceinline__ int route() const { return v.route; }
+    __device__ __forceinline__ CountItem get(int t) const {
+        const int item = items[t], slot = item / v.imax;
+        const int32_t* meta = slot_meta(v, slot);
+        return CountItem{slot_records32(v, slot), slot_records_df(v, slot), slot_records(v, slot),
+                         meta[0] - 1, meta[1], slot_k(v, slot)[item - slot * v.imax]};
     }
-    const double* lay = slot_records(v, slot);
-    const double k = slot_k(v, slot)[j];
-    PairCount r =
-        count_certify_pair(slot_records32(v, slot), slot_records_df(v, slot), lay, N, k, c0, dc,
-                           nlim, half, pair);
-    if (v.route >= 1) r = PairCount{-1, -1, 0};  // test routing: the linear screen from V[0]
-    if (r.cert >= 1) {
-        if (!half) finish_item(v, item, slot, r.cert, c0, dc);
-        return;
+    __device__ __forceinline__ void none(int t) const {
+        const int item = items[t];
+        finish_item(v, item, item / v.imax, -1, c0_, dc_);
     }
-    if (r.n >= 1) {
-        if (search_or_rescan(v, item, slot, lay, N, k, c0, dc, nlim,
-                             TPoint{nlim - 1, -1, 0}, half, pair, active_out))
-            return;
-    } else if (!half) {
-        stt[0] = r.start;
-        stt[1] = r.start > 0 ? 1 : 0;
+    __device__ __forceinline__ void done(int t, int n, int, int) const {
+        const int item = items[t];
+        finish_item(v, item, item / v.imax, n, c0_, dc_);
+    }
+    __device__ __forceinline__ void fallback(int t, int start) const {
+        const int item = items[t], slot = item / v.imax;
+        int32_t* stt = slot_state(v, slot) + 4 * (item - slot * v.imax);
+        stt[0] = start;
+        stt[1] = start > 0 ? 1 : 0;
         stt[2] = PH_SCREEN;
         active_out[atomicAdd(&v.counters[0], 1)] = item;
     }
+    __device__ __forceinline__ void missed(int t, int n, bool from) const { fallback(t, from ? n : 0); }
+};
+
+// Tick, part 0: the batch path's fused counting search and certificate
+// (masw_fused.cuh) for the items admitted since the last tick, G lanes each.
+// A certified item is finished here. The fallback items continue at the next
+// tick with the linear FP32 screen from the end of the pole-free range
+// (carrying the positive sign of count 0) or from V[0], and so do the few that
+// are not certified, from the last point known to have an even count. (300
+// requests of up to 30 layers, 63,660 items: 224 us; a lane pair per item with
+// a double-float count on each lane: 348.)
+template <int G>
+__global__ void __launch_bounds__(128, G == 2 ? 6 : 4) serve_count_kernel(ServeSrc src, int n_items) {
+    count_fused_block<128, G>(src, 0, n_items);
 }
 
 // Tick, part 1 (one warp per active item). PH_SCREEN: up to `chunks` paired
@@ -493,8 +490,16 @@ int tick_launch_impl(masw_server* S, bool* launched) {
     if (cudaMemsetAsync(S->v.counters, 0, 3 * sizeof(int32_t), S->stream) != cudaSuccess)
         return MASW_ECUDA;
     if (n_new) {
-        serve_count_kernel<<<(2 * n_new + 127) / 128, 128, 0, S->stream>>>(
-            S->v, new_items, n_new, S->active[1 - S->cur], S->grid.c0, S->grid.dc);
+        const ServeSrc src{S->v, new_items, S->active[1 - S->cur], S->grid.c0, S->grid.dc};
+        // lanes per item as in the batch path
+        if (n_new <= 4096)
+            serve_count_kernel<32><<<(n_new + 3) / 4, 128, 0, S->stream>>>(src, n_new);
+        else if (n_new <= 16384)
+            serve_count_kernel<8><<<(n_new + 15) / 16, 128, 0, S->stream>>>(src, n_new);
+        else if (n_new <= 24576)
+            serve_count_kernel<4><<<(n_new + 31) / 32, 128, 0, S->stream>>>(src, n_new);
+        else
+            serve_count_kernel<2><<<(n_new + 63) / 64, 128, 0, S->stream>>>(src, n_new);
         if (cudaGetLastError() != cudaSuccess) return MASW_ECUDA;
     }
     if (!prof_mark(S, 2)) return MASW_ECUDA;
