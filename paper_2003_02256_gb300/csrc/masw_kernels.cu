@@ -1969,16 +1969,22 @@ __device__ __forceinline__ double det_rel(const double* __restrict__ lay, int N,
 // A root's bracket narrowed on the FP32 count (inertia_bound_f's recurrence,
 // no bound): [a, bq] inside [lo, hi] with the count's parity changing across
 // it, a few FP32 steps wide, split in three per step by the pair's lanes. The
-// caller checks the FP64 determinant's signs at its ends. Returns false when
-// the FP32 parities at lo and hi agree.
+// caller checks the FP64 determinant's signs at its ends. Returns false unless
+// the count rises by one from lo to hi with no clamped mode between them: a
+// sign change may also be a pole's, and with three roots, or roots and poles,
+// in one grid interval the one taken would depend on the path there.
 static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ lay32, int N,
                                                      float kf, float lo, float hi, int half,
                                                      unsigned pair, float* a_out, float* b_out) {
     float a = lo, bq = hi;
-    int own = inertia_bound_f<false>(lay32, N, kf, half ? bq : a, nullptr) & 1;
-    const int oth = __shfl_xor_sync(pair, own, 1);
-    if (own == oth) return false;
-    const int par_a = half ? oth : own;
+    const float c = half ? bq : a;
+    int own = inertia_bound_f<false>(lay32, N, kf, c, nullptr), j0 = 0;
+    bool sure;
+    for (int j = 0; j < N; ++j)
+        j0 += clamped_modes_bound_f(lay32 + j * LAYER_STRIDE32, kf, c * c, &sure);
+    const int oth = __shfl_xor_sync(pair, own, 1), j0_oth = __shfl_xor_sync(pair, j0, 1);
+    if ((half ? own - oth : oth - own) != 1 || j0 != j0_oth) return false;
+    const int par_a = (half ? oth : own) & 1;
     // down to two FP32 steps of the velocity (2^-22 relative): the count's own
     // error is below that (about 1e-8 relative, from its misses next to roots)
     while (bq - a > 2.4e-7f * bq) {
@@ -2006,10 +2012,10 @@ static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ l
 // a bracket narrower than rel_tol * c, two lanes per item. The bracket is
 // first narrowed on the FP32 count (bracket_root_f32, about 7 FP32 steps) and
 // widened by its error, and kept when the FP64 determinant changes sign
-// across it (else the scan's bracket). Then Illinois (modified
+// across it (else the scan's bracket, with points a quarter tolerance apart
+// throughout). Then Illinois (modified
 // regula falsi) on det K, which has a simple zero there: the secant point x of
-// the bracket ends is evaluated a quarter tolerance on either side (one point
-// per lane); when the two straddle the zero the bracket closes, otherwise the
+// the bracket ends is evaluated a little on either side (one point per lane); when the two straddle the zero the bracket closes, otherwise the
 // nearer point replaces the end of its sign, and an end kept twice in a row
 // has its value halved, so both ends converge. Every 8th step uses the
 // midpoint, so the bracket also shrinks at least as fast as in bisection.
@@ -2018,7 +2024,7 @@ static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ l
 // Bound by the FP64 pipe: from the scan's bracket, closed by points a quarter
 // tolerance apart, it took about 7 pairs of
 // FP64 determinants (2.48 ms for 512 models of 12 layers and 150
-// wavelengths), from the FP32 bracket 2 (1.14 ms).
+// wavelengths), from the FP32 bracket 2 (1.22 ms).
 __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __restrict__ layers32,
                                                      const int32_t* __restrict__ idx,
                                                      double rel_tol, double* croot) {
@@ -2091,7 +2097,7 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __
             double x = (i % 8 == 7) ? 0.5 * (lo + hi) : hi - f_hi * (hi - lo) / (f_hi - f_lo);
             if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
             const double w = hi - lo, slope = (f_hi - f_lo) / w;
-            const double eps = fmax(0.25 * rel_tol * hi, 1e-3 * w);
+            const double eps = narrow ? fmax(0.25 * rel_tol * hi, 1e-3 * w) : 0.25 * rel_tol * hi;
             const double p0 = fmax(x - eps, lo + 0.25 * (x - lo));
             const double p1 = fmin(x + eps, hi - 0.25 * (hi - x));
             const double fp = det_rel(lay, N, k, half ? p1 : p0, e_ref);
@@ -2109,7 +2115,7 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __
                 // taken when that is below a tenth of the tolerance (with
                 // side 0 both slopes are the determinant's).
                 const double v = hi - lo, s1 = (f1 - f0) / v;
-                if (side == 0 && fabs(s1 - slope) * v * v < 0.4 * rel_tol * hi * w * fabs(s1)) {
+                if (narrow && side == 0 && fabs(s1 - slope) * v * v < 0.4 * rel_tol * hi * w * fabs(s1)) {
                     result = hi - f1 / s1;
                     break;
                 }
