@@ -17,6 +17,24 @@ import torch
 from . import masw
 
 
+def _model_index(batch, dev):
+    """The model of every record and of every thickness, laid out on ``dev`` once
+    per batch (its layer counts are fixed): an upload in each forward pass would
+    wait there for the whole evaluation."""
+    per_dev = batch.__dict__.setdefault("_model_index", {})
+    index = per_dev.get(dev)
+    if index is None:
+        nl = np.asarray(batch.models.n_layers, dtype=np.int64)
+        with torch.inference_mode(False):  # later passes may save them for backward
+            index = tuple(torch.as_tensor(np.repeat(np.arange(nl.size), n), device=dev)
+                          for n in (nl + 1, nl))
+        per_dev[dev] = index
+    if dev.type == "cuda":  # in use on this stream beyond the batch's own life
+        for t in index:
+            t.record_stream(torch.cuda.current_stream(dev))
+    return index
+
+
 class MaswMisfit(torch.autograd.Function):
     @staticmethod
     def forward(ctx, beta, h, batch, ce, kind=masw.MISFIT_LSQ, sigma=2.0):
@@ -31,9 +49,7 @@ class MaswMisfit(torch.autograd.Function):
         gb = torch.empty_like(b)
         gh = torch.empty(max(hh.numel(), 1), dtype=torch.float64, device=dev)
         masw.misfit_grad(batch.handle, ce_t, kind, sigma, phi, gb, gh)
-        nl = np.asarray(batch.models.n_layers, dtype=np.int64)
-        rec_model = torch.as_tensor(np.repeat(np.arange(nl.size), nl + 1), device=dev)
-        h_model = torch.as_tensor(np.repeat(np.arange(nl.size), nl), device=dev)
+        rec_model, h_model = _model_index(batch, dev)
         ctx.save_for_backward(gb, gh[:hh.numel()], rec_model, h_model)
         return phi
 

@@ -67,9 +67,11 @@ struct masw_batch {
     int32_t* d_search_order = nullptr;
     int64_t* d_grad_off = nullptr;
     int32_t* d_counter = nullptr;
+    // results: ct, then idx and status in the same allocation (curves_out)
     double* d_ct = nullptr;
     int32_t* d_idx = nullptr;
     int32_t* d_status = nullptr;
+    std::vector<double> h_out;  // their host copy for small batches
     // lazily allocated
     double* d_croot = nullptr;
     double* d_rows = nullptr;
@@ -174,6 +176,16 @@ static bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+static bool is_pageable_ptr(const void* p) {
+    cudaPointerAttributes a;
+    if (!p) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return a.type == cudaMemoryTypeUnregistered;
+}
+
 // masw_test_fail_alloc: ordinal of the next device allocation to fail (-1: none)
 static std::atomic<int> g_alloc_fail_at{-1};
 
@@ -233,6 +245,9 @@ static int copy_in(T* dst, const T* src, size_t n, cudaStream_t s) {
     if (kind == cudaMemcpyHostToDevice) CK(cudaStreamSynchronize(s));  // caller may reuse src
     return MASW_OK;
 }
+
+// Items up to which pageable results come in one copy (64 KB).
+constexpr size_t STAGED_ITEMS = 4096;
 
 static double grid_v(const masw_grid& g, int n) { return std::fma((double)n, g.dc, g.c0); }
 
@@ -339,7 +354,7 @@ static void free_batch(masw_batch* B) {
     void* ptrs[] = {B->d_layers, B->d_loff,  B->d_woff,  B->d_nlim,   B->d_k,
                     B->d_item_model, B->d_order_sorted, B->d_order_natural, B->d_search_order,
                     B->d_grad_off,
-                    B->d_counter, B->d_ct, B->d_idx, B->d_status, B->d_croot, B->d_rows, B->d_bs,
+                    B->d_counter, B->d_ct, B->d_croot, B->d_rows, B->d_bs,
                     B->d_dphi, B->d_ce, B->d_misfit, B->d_gb, B->d_gh, B->d_layers32, B->d_layers_df,
                     B->d_n32, B->d_cert, B->d_search, B->d_unres, B->d_fallback, B->d_counters,
                     B->d_nsearch, B->d_one, B->d_two, B->d_search2, B->d_unres2, B->d_fallback2, B->d_upd, B->d_upd_err,
@@ -628,7 +643,7 @@ int masw_model_batch_create(const masw_models_desc* md, const masw_grid* grid, v
         dev_alloc(&B->d_order_sorted, nw) || dev_alloc(&B->d_order_natural, nw) ||
         dev_alloc(&B->d_search_order, nw) ||
         dev_alloc(&B->d_grad_off, nw + 1) || dev_alloc(&B->d_counter, 1) ||
-        dev_alloc(&B->d_ct, nw) || dev_alloc(&B->d_idx, nw) || dev_alloc(&B->d_status, nw) ||
+        dev_alloc(&B->d_ct, 2 * nw) ||
         dev_alloc(&B->d_layers32, rec32.size()) || dev_alloc(&B->d_layers_df, recdf.size()) ||
         dev_alloc(&B->d_n32, nw) || dev_alloc(&B->d_cert, nw) ||
         dev_alloc(&B->d_search, nw) || dev_alloc(&B->d_unres, nw) || dev_alloc(&B->d_fallback, nw) ||
@@ -639,6 +654,9 @@ int masw_model_batch_create(const masw_models_desc* md, const masw_grid* grid, v
         free_batch(B);
         return MASW_ENOMEM;
     }
+    B->d_idx = reinterpret_cast<int32_t*>(B->d_ct + nw);
+    B->d_status = B->d_idx + nw;
+    if (nw <= STAGED_ITEMS) B->h_out.resize(2 * nw);
     auto up = [&](void* d, const void* s, size_t bytes) {
         return bytes ? cudaMemcpy(d, s, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
     };
@@ -768,13 +786,34 @@ int masw_batch_info(const masw_batch* B, int64_t* n_items, int32_t* n_models, in
     return MASW_OK;
 }
 
+// The curves to the caller's buffers. A copy to pageable host memory blocks
+// for about 8 us whatever its size, so those of a small batch come in one.
+static int curves_out(masw_batch* B, double* ct, int32_t* idx, int32_t* status, bool* need_sync) {
+    const size_t n = (size_t)B->n_items;
+    if (n && !B->h_out.empty() && is_pageable_ptr(ct) && is_pageable_ptr(idx) &&
+        is_pageable_ptr(status)) {
+        CK(cudaMemcpyAsync(B->h_out.data(), B->d_ct, 2 * n * sizeof(double), cudaMemcpyDeviceToHost,
+                           B->stream));
+        CK(cudaStreamSynchronize(B->stream));
+        const double* h = B->h_out.data();
+        std::memcpy(ct, h, n * sizeof(double));
+        std::memcpy(idx, h + n, n * sizeof(int32_t));
+        std::memcpy(status, reinterpret_cast<const int32_t*>(h + n) + n, n * sizeof(int32_t));
+        *need_sync = false;
+        return MASW_OK;
+    }
+    int rc;
+    if ((rc = copy_out(ct, B->d_ct, n, B->stream, need_sync)) ||
+        (rc = copy_out(idx, B->d_idx, n, B->stream, need_sync)) ||
+        (rc = copy_out(status, B->d_status, n, B->stream, need_sync)))
+        return rc;
+    return MASW_OK;
+}
+
 static int finish_outputs(masw_batch* B, double* ct, int32_t* idx, int32_t* status) {
     bool sync = false;
     int rc;
-    if ((rc = copy_out(ct, B->d_ct, B->n_items, B->stream, &sync)) ||
-        (rc = copy_out(idx, B->d_idx, B->n_items, B->stream, &sync)) ||
-        (rc = copy_out(status, B->d_status, B->n_items, B->stream, &sync)))
-        return rc;
+    if ((rc = curves_out(B, ct, idx, status, &sync))) return rc;
     if (sync) CK(cudaStreamSynchronize(B->stream));
     return MASW_OK;
 }
@@ -1064,9 +1103,7 @@ int masw_misfit_curves(masw_batch* B, const double* ce, int32_t kind, double sig
     if ((rc = run_scan(B))) return rc;
     CK(launch_misfit(B->dev(false), B->d_ct, B->d_ce, kind, sigma, B->d_misfit, nullptr, B->stream));
     if ((rc = copy_out(misfit, B->d_misfit, B->n_models, B->stream, &sync)) ||
-        (rc = copy_out(ct, B->d_ct, B->n_items, B->stream, &sync)) ||
-        (rc = copy_out(ct_idx, B->d_idx, B->n_items, B->stream, &sync)) ||
-        (rc = copy_out(status, B->d_status, B->n_items, B->stream, &sync)))
+        (rc = curves_out(B, ct, ct_idx, status, &sync)))
         return rc;
     if (sync) CK(cudaStreamSynchronize(B->stream));
     return MASW_OK;
