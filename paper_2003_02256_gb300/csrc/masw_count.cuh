@@ -7,27 +7,21 @@
 //    function of the grid index, 0 at c = 0 (Wittrick-Williams below the
 //    lowest clamped-layer mode). One thread bisects it (count_search_single,
 //    or count_search_guess from a guess interpolated between the indices of
-//    neighbouring wavelengths),
-//    or a pair of lanes evaluates the top of the range and its midpoint, then
-//    splits the bracket in three per step, one point per lane (the fused
-//    kernel and the serving tick, where the certificate's lanes follow):
-//    about log2(npf), or log3(npf) steps, instead of Algorithm 1's linear
-//    walk. The first nonzero point goes to the certificate whatever its FP32
-//    parity.
-//  * Certificate (a pair of adjacent lanes; the recurrence over
-//    double-float elements, det_inertia_dd in masw_df.cuh: the Schur step in
-//    double-float too, the half-space's in FP64; points above the pole-free
-//    range take det_inertia_df, the FP64 step). The count is 0 at V[n-1] (so
-//    0, and V[0]'s sign, at every point below) and odd at V[n] (the sign
-//    differs).
-//    When the FP32 count was off by one next to the change (count 0 at both
-//    points: the change is higher; nonzero at V[n-1]: lower), the pair takes
-//    one FP64 step of two points in that direction, inside the range. An
-//    even FP64 count (two or more) after count 0 means no sign change there:
-//    a second search looks for the first odd count above it, certified the
-//    same way. Items left without a certificate fall back: the batch path
-//    searches the FP64 mode count s + 2 J0 from V[0] (masw_modes.cuh), the
-//    serving tick scans linearly from `start`.
+//    neighbouring wavelengths), or G lanes split the bracket in G + 1 per step
+//    (the _group forms): about log2(npf), or log_{G+1}(npf) steps, instead of
+//    Algorithm 1's linear walk.
+//  * Certificate. The count is 0 at V[n-1] (so 0, and V[0]'s sign, at every
+//    point below) and odd at V[n] (the sign differs). The search evaluates
+//    these two counts with their FP32 error bound (masw_bound.cuh); the ones
+//    it does not prove are evaluated in double-float (det_inertia_dd in
+//    masw_df.cuh, the half-space's step in FP64). When the FP32 count was off
+//    next to the change (count 0 at both points: the change is higher;
+//    nonzero at V[n-1]: lower), a few double-float points in that direction,
+//    inside the range, settle it. An even count (two or more) after count 0
+//    means no sign change there: a second search looks for the first odd count
+//    above it, certified the same way. Items left without a certificate take
+//    the sign scan (batch path) or the linear screen (serving tick) from the
+//    last point known to have an even count.
 #pragma once
 
 #include "masw_bound.cuh"
@@ -105,11 +99,10 @@ __device__ __forceinline__ int count_bound_at(const float* __restrict__ lay32, i
     return inertia_bound_f(lay32, N, kf, (float)grid_c(c0, dc, n), sure);
 }
 
-// The search stage by one thread (the split search kernel): the first grid
-// point in [0, npf) with a nonzero FP32 count, or -1, by bisection. One point
-// per step is one bit per evaluation, against log2(3)/2 for a pair's three-way
-// split, so an item takes about 20 % fewer evaluations; the pair form stays
-// where the certificate's lanes follow in the same kernel. The bisection's
+// The search stage by one thread (the split search kernel on large batches):
+// the first grid point in [0, npf) with a nonzero FP32 count, or -1, by
+// bisection. One point per step is one bit per evaluation, the fewest; lane
+// groups take fewer steps where latency counts. The bisection's
 // points take the plain count and the two points of the result the bounded
 // one: about 10 + 2 evaluations, the bounded one costing 1.5 plain ones.
 __device__ __forceinline__ Located count_search_single(const float* __restrict__ lay32, int N,

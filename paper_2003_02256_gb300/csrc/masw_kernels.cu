@@ -15,12 +15,14 @@
 //                         FP64 check on the Wittrick-Williams mode count.
 //  count_search_kernel,   precision 2 (default): FP32 search on the
 //  count_certify_kernel   negative-eigenvalue count below the pole-free bound
-//                         (one thread per item, bisection, two passes: every
-//                         6th wavelength of a model first, then the others
-//                         from a guess on the line through their neighbours'
-//                         indices) and its FP64
-//                         certificate, a lane pair per item; for small batches
-//                         both in one kernel (lane pairs, plan count_split).
+//                         (bisection, two passes: every 6th wavelength of a
+//                         model first, then the others from a guess on the
+//                         line through their neighbours' indices), with an
+//                         error bound that proves most of the counts its
+//                         certificate needs; the other counts in double-float
+//                         from lists.
+//  count_fused_kernel     the same for smaller batches in one kernel, lane
+//                         groups per item (plan count_split 0).
 //                         The fallback items take fallback32_kernel (linear
 //                         FP32 scan) and verify64_list_kernel (the check), for
 //                         large batches on a second stream beside the
@@ -540,38 +542,20 @@ struct CountLists {
 constexpr int32_t ONE_LOW = 1 << 30;    // list `one`: V[n-1] is the point wanted
 constexpr int32_t SCAN_FROM = 1 << 30;  // search list: the count is even up to V[n32[item]]
 
-// The counting search's FP64 certificate (plan precision 2), two lanes per
-// item (certify_pair; natural item order, or by layer count over a whole
-// batch: a warp's 16 items share a model and have adjacent wavelengths, so
-// their branches agree), with the search in the same kernel (count_search_pair,
-// small batches) or before it (SPLIT: its index in nsearch). Items whose
-// change lies above the pole-free range or at V[0] go to the fallback list
-// (linear FP32 scan and mode-count check); the certificate's own failures
-// (the counts around the located point, or an even count with no odd one
-// found above it) to the sign scan's list. Certified items keep SCREEN_COUNTED in n32. B threads per
-// block (plan count_block: 64, 128 or 256), each block's B/2 items
-// consecutive, so its warps share the records of one or two models in L1;
-// the launch bounds ask for 896 resident threads per SM (at most 73
-// registers a thread) for B = 64 and 128, and 512 for 256 (128 registers, no
-// spills: the default beside the second stream, whose chain then finds room
-// sooner); with SPLIT (plan count_split: the search ran before in
-// count_search_kernel, its index in n32), 640 for B = 64 (96 registers,
-// fewer spills), so that the block size also picks among the register
-// budgets.
-// Search stage alone (count_search_single or count_search_guess, one
-// thread per item), with what its FP32 counts' error bound proves. An item
+// Search stage of the split plans (count_search_single or
+// count_search_guess, G lanes per item), with what its FP32 counts' error
+// bound proves. An item
 // whose counts at V[n-1] (0) and V[n] (odd) are both proven is finished here.
 // With one of them proven it joins the list `one`, with none the list `two`
 // (count_certify_kernel). Bound by instruction issue (FP32, 88 % of cycles in
 // the first pass on the 8192-model ragged batch).
-// The items the certificate would only pass on to
-// the linear FP32 scan (no count change inside the pole-free range, a mode
+// The items the certificate would only pass on to the
+// linear FP32 scan (no count change inside the pole-free range, a mode
 // below V[0], test routing 1..3) go straight to that list with their start in
 // n32, and nsearch gets 0 for them and for models without a scan range
 // (results written here), so that the fallback chain can run on a second
 // stream beside the certificate. Natural item order: a warp's 32 items share
 // a model or two and have adjacent wavelengths, so their branches agree.
-// G lanes per item (a group search where G > 1).
 // PASS 0: the items [item_begin, item_end) in natural order; 1: the anchor
 // items of b.search_order (every SEARCH_STRIDE-th wavelength of a model and
 // its last), each searched in full; 2: the other items, each searched
@@ -742,6 +726,11 @@ struct BatchSrc {
 // an item whose count there is not the certificate's (an FP32 index off by
 // one, or an even count). The pairs of w.two come first: theirs is the longer
 // work.
+// Bound by instruction issue and fetch (the double-float element is about
+// 1,300 instructions a layer). B threads per block (plan count_block): 2 blocks
+// of 256 per SM (128 registers, no spills) or 7 of 128 or 10 of 64. On the
+// 8192-model ragged batch 0.55 ms, where counts in double-float at both points
+// of every item took 4.6 ms.
 template <int B>
 __global__ void __launch_bounds__(B, (B == 256 ? 2 : B == 64 ? 10 : 7))
     count_certify_kernel(DevBatch b, const float* __restrict__ layers32, ScanOut o, CountLists w,
