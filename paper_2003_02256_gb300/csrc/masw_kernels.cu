@@ -407,15 +407,25 @@ __global__ void verify64_kernel(DevBatch b, ScanOut o, const int32_t* __restrict
     verify_item(b, o, item, n32[item], search, n_search);
 }
 
+// First statement of the tail's kernels (launch_prio, early): waits for the
+// kernel before to end, then lets the next one's blocks come in. Five kernels
+// over lists that are often empty cost little but their launches. What
+// the kernels before write is not __restrict__ here: loads through such a
+// pointer may be moved above the wait or come from a stale cache line.
+__device__ __forceinline__ void after_previous() {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+
 // The same check over a device-counted list (the fallback items of the
 // counting search), four lanes per item so that its three FP64 evaluations
 // run side by side (a lone evaluation is a long dependent FP64 chain; a few
 // listed items are latency-bound), grid-stride over the list.
-__global__ void __launch_bounds__(128) verify64_list_kernel(DevBatch b, ScanOut o,
-                                                            const int32_t* __restrict__ n32,
-                                                            const int32_t* __restrict__ list,
-                                                            const int32_t* __restrict__ n_list,
+__global__ void __launch_bounds__(128) verify64_list_kernel(DevBatch b, ScanOut o, const int32_t* n32,
+                                                            const int32_t* list,
+                                                            const int32_t* n_list,
                                                             int32_t* search, int32_t* n_search) {
+    after_previous();
     const int total = *n_list;
     const int lane = threadIdx.x & 31;
     const int sub = lane & 3;
@@ -459,9 +469,10 @@ __global__ void __launch_bounds__(128) verify64_list_kernel(DevBatch b, ScanOut 
 // sign of an even negative-eigenvalue count). The first change of a round is the smallest index any warp
 // found; warp w's first point compares with warp w-1's last.
 __global__ void __launch_bounds__(256) fallback32_kernel(DevBatch b, const float* __restrict__ layers32,
-                                                         int32_t* n32, const int32_t* __restrict__ fallback,
-                                                         const int32_t* __restrict__ n_fallback,
+                                                         int32_t* n32, const int32_t* fallback,
+                                                         const int32_t* n_fallback,
                                                          int32_t* counter, int stage_layers) {
+    after_previous();
     extern __shared__ float smemf[];
     __shared__ int s_item, s_res, s_last[32];
     const int lane = threadIdx.x & 31;
@@ -831,10 +842,11 @@ __global__ void __launch_bounds__(B, (B == 256 ? 2 : (G == 2 ? 768 : 512) / B))
 // count alone.
 __global__ void __launch_bounds__(32) first_count64_kernel(DevBatch b, ScanOut o, int32_t* n32,
                                                            const float* __restrict__ layers32,
-                                                           const int32_t* __restrict__ list,
-                                                           const int32_t* __restrict__ n_list,
+                                                           const int32_t* list,
+                                                           const int32_t* n_list,
                                                            int32_t* counter, int32_t* unresolved,
                                                            int32_t* n_unresolved) {
+    after_previous();
     const int half = threadIdx.x & 1;
     const unsigned pair = 3u << (threadIdx.x & 30);
     const int total = *n_list;
@@ -890,9 +902,10 @@ constexpr int SIGN_SCAN_THREADS = 128;
 constexpr int SIGN_SCAN_BUDGET = 1024;
 __global__ void __launch_bounds__(SIGN_SCAN_THREADS, 4)
     sign_scan_kernel(DevBatch b, ScanOut o, const float* __restrict__ layers32, int32_t* n32,
-                     const int32_t* __restrict__ list, const int32_t* __restrict__ n_list,
+                     const int32_t* list, const int32_t* n_list,
                      int32_t* counter, int32_t* hard, int32_t* n_hard, int32_t* unresolved,
                      int32_t* n_unresolved) {
+    after_previous();
     __shared__ float s_lay[32 * LAYER_STRIDE32];  // records of up to 31 layers
     __shared__ int s_item, s_first, s_open, s_bad, s_end[2];
     __shared__ int s_list[SIGN_SCAN_THREADS];
@@ -992,9 +1005,10 @@ __global__ void __launch_bounds__(SIGN_SCAN_THREADS, 4)
 // monotone at the evaluated points): Algorithm 1 in FP64 from V[0], one warp
 // per item, 32 points per chunk.
 __global__ void __launch_bounds__(256) resolve64_kernel(DevBatch b, ScanOut o,
-                                                        const int32_t* __restrict__ unresolved,
-                                                        const int32_t* __restrict__ n_unresolved,
+                                                        const int32_t* unresolved,
+                                                        const int32_t* n_unresolved,
                                                         int32_t* counter) {
+    after_previous();
     const int lane = threadIdx.x & 31;
     const int total = *n_unresolved;
     if (total == 0) return;  // the usual case: no atomics on the queue
@@ -1026,20 +1040,27 @@ __global__ void __launch_bounds__(256) resolve64_kernel(DevBatch b, ScanOut o,
 }
 
 // Launch with an explicit priority (cudaLaunchAttributePriority, kept as the
-// node's priority when captured into a graph); prio 0 launches plainly.
+// node's priority when captured into a graph), and optionally early: the
+// kernel's blocks take their places while the kernel before it in the stream
+// still runs, and wait for its end in after_previous().
 template <typename... Arg, typename... Act>
 static cudaError_t launch_prio(void (*kernel)(Arg...), int grid, int block, size_t shm,
-                               cudaStream_t s, int prio, Act&&... args) {
+                               cudaStream_t s, int prio, bool early, Act&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = shm;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributePriority;
-    at[0].val.priority = prio;
+    cudaLaunchAttribute at[2];
+    if (prio != 0) {  // 0: the stream's own priority
+        at[cfg.numAttrs].id = cudaLaunchAttributePriority;
+        at[cfg.numAttrs++].val.priority = prio;
+    }
+    if (early) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
     cfg.attrs = at;
-    cfg.numAttrs = prio != 0 ? 1 : 0;  // 0: the stream's own priority
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Act>(args)...);
 }
 
@@ -1048,20 +1069,24 @@ static cudaError_t launch_prio(void (*kernel)(Arg...), int grid, int block, size
 // check, then the sign scan of the items that failed a check, the mode-count
 // search of those it hands on and the
 // FP64 re-scan of the items whose counts failed. phase_ev1: recorded after
-// the search (or nullptr).
+// the search (or nullptr). early: each kernel's blocks come in while the one
+// before still runs (64,000 items without a graph: 194 -> 181 us); not beside a
+// second stream, whose blocks would wait for the places that they hold (701
+// models with one: 747 -> 781 us).
 static cudaError_t launch_tail(const DevBatch& b, const ScanOut& o, const ScanPlan& p,
                                const float* layers32, int32_t* n32, int32_t* search,
                                int32_t* unresolved, int32_t* fallback, int32_t* counters,
                                int counting, int n, cudaStream_t s, int prio,
-                               cudaEvent_t phase_ev1) {
+                               cudaEvent_t phase_ev1, bool early) {
     cudaError_t e;
     if (counting) {
         e = launch_prio(fallback32_kernel, std::max(1, std::min(p.blocks, n)), 256,
-                        (size_t)p.stage_layers * LAYER_STRIDE32 * sizeof(float), s, prio, b,
+                        (size_t)p.stage_layers * LAYER_STRIDE32 * sizeof(float), s, prio, false, b,
                         layers32, n32, fallback, counters + 3, counters + 4, p.stage_layers);
         if (e != cudaSuccess) return e;
         e = launch_prio(verify64_list_kernel, std::max(1, std::min(p.blocks, (4 * n + 127) / 128)),
-                        128, 0, s, prio, b, o, n32, fallback, counters + 3, search, counters + 5);
+                        128, 0, s, prio, early, b, o, n32, fallback, counters + 3, search,
+                        counters + 5);
         if (e != cudaSuccess) return e;
     }
     // The mode-count search and the FP64 re-scan work through short lists
@@ -1073,15 +1098,15 @@ static cudaError_t launch_tail(const DevBatch& b, const ScanOut& o, const ScanPl
     // (the fallback list is done with: it takes the items handed on)
     int32_t* const hard = fallback;
     e = launch_prio(sign_scan_kernel, std::max(1, std::min(4 * sms, n)), SIGN_SCAN_THREADS, 0, s,
-                    prio, b, o, layers32, n32, search, counters + 5, counters + 6, hard,
+                    prio, early && counting, b, o, layers32, n32, search, counters + 5, counters + 6, hard,
                     counters + 9, unresolved, counters + 1);
     if (e != cudaSuccess) return e;
-    e = launch_prio(first_count64_kernel, lblocks, 32, 0, s, prio, b, o, n32, layers32, hard,
+    e = launch_prio(first_count64_kernel, lblocks, 32, 0, s, prio, early, b, o, n32, layers32, hard,
                     counters + 9, counters + 10, unresolved, counters + 1);
     if (e != cudaSuccess) return e;
     if (phase_ev1 && (e = cudaEventRecord(phase_ev1, s)) != cudaSuccess) return e;
-    return launch_prio(resolve64_kernel, lblocks, 32, 0, s, prio, b, o, unresolved, counters + 1,
-                       counters + 2);
+    return launch_prio(resolve64_kernel, lblocks, 32, 0, s, prio, early && !phase_ev1, b, o, unresolved,
+                       counters + 1, counters + 2);
 }
 
 cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPlan& p,
@@ -1157,7 +1182,7 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
             if ((e = cudaEventRecord(side->fork, s)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(side->s, side->fork, 0)) != cudaSuccess) return e;
             e = launch_tail(b, o, p, layers32, n32, side->search, side->unresolved, side->fallback,
-                            side_counters, 1, n, side->s, side->prio, nullptr);
+                            side_counters, 1, n, side->s, side->prio, nullptr, false);
             if (e != cudaSuccess) return e;
             if ((e = cudaEventRecord(side->join, side->s)) != cudaSuccess) return e;
         }
@@ -1225,7 +1250,7 @@ cudaError_t launch_screen_scan(const DevBatch& b, const ScanOut& o, const ScanPl
     // the certificate's own failures (with overlap: no fallback items here;
     // all of them otherwise)
     e = launch_tail(b, o, p, layers32, n32, search, unresolved, fallback, counters,
-                    counting && !overlap, n, s, 0, phase_ev ? phase_ev[1] : nullptr);
+                    counting && !overlap, n, s, 0, phase_ev ? phase_ev[1] : nullptr, !overlap);
     if (e != cudaSuccess) return e;
     if (overlap && (e = cudaStreamWaitEvent(s, side->join, 0)) != cudaSuccess) return e;
     return cudaSuccess;
