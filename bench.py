@@ -79,11 +79,6 @@ def make_workload(name: str, n_models: int, rank: int = 0):
 # Every FP64 kernel runs this arithmetic; it is the per-unit figure of the
 # rooflines below.
 F_LAYER_FLOPS = 149.1
-# FP64 flops the counting kernel executes per layer-evaluation now that the
-# element runs in double-float on the FP32 pipe and only the Schur step (and
-# the exact conversions) on the FP64 pipe: 55.6 M DFMA, 57.6 M DMUL, 39.9 M
-# DADD over the same 3,686,400 layer-evaluations (ncu; profiles/).
-F_LAYER_FLOPS_EXECUTED64 = 56.6
 # FP32 flops per layer-evaluation of the screen kernel (2*FFMA + FMUL + FADD
 # per executed (layer, c) pair: 29.6 FFMA, 54.2 FMUL, 16.4 FADD; ncu
 # instruction counters of the 64-model case, profiles/).
@@ -97,26 +92,19 @@ FP32_FFMA_PER_CLK_SM = 128.0
 # the maximum SM clock.
 FP64_DFMA_PER_CLK_SM = 2.0
 SM_MAX_MHZ = 2070.0
-# DRAM bytes (read + write) of one count_certify launch, from ncu captures
-# (dram__bytes_read.sum + dram__bytes_write.sum) of the full workload, as
-# (bytes, models of that launch); the records, wavenumbers, item tables and
-# the search's indices are read once. Scaled by the models of a launch; None
-# where no capture of the current kernel exists.
-# uniform: 5.27 MB for the 1024-model launch of count_certify_kernel<128,
-# true> (most of its outputs stay in L2); ragged: 49.51 MB for the
-# 8192-model launch of count_certify_kernel<256, true> (47.71 MB read,
-# 1.80 MB written by the end of the launch).
-CERTIFY_DRAM_BYTES = {"uniform": (5.355264e6, 1024), "ragged": (49.506048e6, 8192)}
-# Warp instructions a kernel issues per layer-evaluation (ncu
-# smsp__inst_executed.sum of one full-workload launch / its layer-evaluations
-# counted as in counting_evals), by workload: the certificate kernel per
-# certificate layer-evaluation, the search kernels (both passes) per FP32
-# one. A kernel's ceiling is the SM's issue rate, ISSUE_PER_CLK_SM warp
-# instructions per clock, over this count.
-CERTIFY_WARP_INSTR_PER_LAYER_EVAL = {"uniform": 51.25, "ragged": 51.95}
+# DRAM bytes (read + write) of the search's two launches of one scan, from ncu
+# captures (dram__bytes_read.sum + dram__bytes_write.sum) of the full workload,
+# as (bytes, models of that launch); the records, wavenumbers and item tables
+# are read once a launch. Scaled by the models of a launch.
+SEARCH_DRAM_BYTES = {"uniform": (7.245e6, 1024), "ragged": (160.64e6, 8192)}
 # the split search's anchor stride (SEARCH_STRIDE in csrc/masw_internal.h)
 SEARCH_STRIDE = 6
-SEARCH_WARP_INSTR_PER_LAYER_EVAL = {"uniform": 8.61, "ragged": 8.21}
+# Warp instructions the search kernels (both passes, the bounded counts next
+# to the change included) issue per FP32 layer-evaluation of
+# split_search_evals (ncu smsp__inst_executed.sum of one full-workload scan),
+# by workload. The ceiling is the SM's issue rate, ISSUE_PER_CLK_SM warp
+# instructions per clock, over this count.
+SEARCH_WARP_INSTR_PER_LAYER_EVAL = {"uniform": 12.41, "ragged": 11.57}
 ISSUE_PER_CLK_SM = 4
 # Warp instructions per layer-evaluation of the leaky continuation's scan
 # kernel, element and Schur step in double-float (ncu smsp__inst_executed.sum
@@ -465,9 +453,11 @@ def counting_evals(models, grid, idx, st, nlim, n32, split=True):
     """Per-item evaluations of the counting-search scan (plan precision 2).
     FP32 layer evaluations of the search, npf = grid points below the
     pole-free bound min_i beta_i sqrt(1 + (pi/(k h_i))^2): split (its own
-    kernels, one thread per item) as split_search_evals; fused (a lane pair)
-    1 + ceil(log3 npf) steps of two inertia counts. FP64 layer evaluations of
-    the certificate: 2 per counted item. Fallback items: the linear FP32
+    kernels, one thread per item) as split_search_evals; fused (G lanes per
+    item, G = 32 / 8 / 4 / 2 by the batch's items) ceil(log_{G+1} npf) steps of
+    G inertia counts and two with the error bound. The certificate's counts: 2
+    per counted item; the bound proves most of them in the search, so this is
+    what they come to if all were evaluated. Fallback items: the linear FP32
     scan from its start up to the change, and the three-point FP64 check."""
     counted = (n32 >= 0) & ((n32 & (1 << 30)) != 0)
     item_model = np.repeat(np.arange(models.n_models), models.n_lambda)
@@ -486,8 +476,10 @@ def counting_evals(models, grid, idx, st, nlim, n32, split=True):
     if split:
         search = split_search_evals(models, npf, root)
     else:
-        steps = np.where(npf >= 2, 1 + np.ceil(np.log(np.maximum(npf, 2)) / np.log(3.0)), 1)
-        search = np.where(npf >= 1, 2 * steps, 0)
+        n = models.n_items
+        lanes = 32 if n <= 4096 else 8 if n <= 16384 else 4 if n <= 24576 else 2
+        steps = np.ceil(np.log(np.maximum(npf, 2)) / np.log(lanes + 1.0))
+        search = np.where(npf >= 1, lanes * steps + 2, 0)
     start = np.where(root >= npf, npf, 0)
     linear = np.where(counted, 0, np.maximum(root - start + 1, 0))
     live = lim >= 2
@@ -498,57 +490,46 @@ def counting_evals(models, grid, idx, st, nlim, n32, split=True):
 
 
 def counting_roofline(models, grid, idx, st, nlim, n32, phases, peak64, micro, sms, workload):
-    """Roofline of the dominant kernel of a counting-search scan, the FP64
-    certificate (count_certify_kernel; with the fused plan, the search runs
-    inside it): its FP64 work (2 layer-evaluation chains per counted item)
-    against the FP64 pipe, from algorithmic layer evaluations / device time.
-    The FP32 search's work is reported against the FP32 pipe, over its own
-    kernel's time when it has one. Also the linear scan's count (Algorithm
-    1's (idx + 1)(N + 1) layer-evaluations per item) and how much of it the
-    counting search leaves out."""
+    """Roofline of the dominant kernel of a counting-search scan, the FP32
+    search (count_search_kernel, both passes; with the fused plan
+    count_fused_kernel, certificate included): its FP32 layer-evaluations /
+    device time against the SM's instruction issue for its measured
+    instruction mix (the FP32 pipe where that was not measured). The bounded
+    counts next to the change prove most certificates; the certificate kernel
+    after it completes the others in double-float. Also the linear scan's
+    count (Algorithm 1's (idx + 1)(N + 1) layer-evaluations per item) and how
+    much of it the counting search leaves out."""
     split = phases[3] is not None
     e32, e64, e64_fb, frac_counted = counting_evals(models, grid, idx, st, nlim, n32, split)
     linear = algorithmic_layer_evals(models, idx, st, nlim)
     peak32 = FP32_FFMA_PER_CLK_SM * 2.0 * sms * SM_MAX_MHZ * 1e6
-    t0 = (phases[4] if split else phases[0]) * 1e-3
-    t32 = (phases[3] if split else phases[0]) * 1e-3
-    achieved = e64 * F_LAYER_FLOPS / t0
-    cap = CERTIFY_DRAM_BYTES.get(workload)
-    wi = CERTIFY_WARP_INSTR_PER_LAYER_EVAL.get(workload) if split else None
-    # the roof: the FP64 pipe for the plain FP64 element and step, the SM's
-    # instruction issue for the double-float form (its instruction mix
-    # measured by ncu); both in the algorithmic flops of a layer-evaluation
-    peak_issue = (ISSUE_PER_CLK_SM * sms * SM_MAX_MHZ * 1e6 / wi * F_LAYER_FLOPS) if wi else None
-    roof = peak_issue if peak_issue else peak64
-    kernel = ("count_certify_kernel (FP64 certificate: double-float element on the FP32 pipe, "
-              "Schur step on the FP64 pipe; the FP32 search in count_search_kernel before it)"
-              if split else
-              "count_certify_kernel (FP64 certificate: double-float element on the FP32 pipe, "
-              "Schur step on the FP64 pipe; FP32 search alongside)")
+    t0 = (phases[3] if split else phases[0]) * 1e-3
+    achieved = e32 * F_LAYER_FLOPS_FP32 / t0
+    cap = SEARCH_DRAM_BYTES.get(workload) if split else None
+    wi = SEARCH_WARP_INSTR_PER_LAYER_EVAL.get(workload) if split else None
+    peak_issue = (ISSUE_PER_CLK_SM * sms * SM_MAX_MHZ * 1e6 / wi * F_LAYER_FLOPS_FP32) if wi else None
+    roof = peak_issue if peak_issue else peak32
+    kernel = ("count_search_kernel (FP32 search and error bound, two passes; the open "
+              "certificates in count_certify_kernel after it)" if split else
+              "count_fused_kernel (FP32 search with its error bound, open certificates in "
+              "double-float in the same kernel)")
     return {"bound": "alu", "unit": "TFLOP/s",
             "achieved": achieved / 1e12, "peak": roof / 1e12, "frac": achieved / roof,
             "traffic": None if cap is None else cap[0] * models.n_models / cap[1],
             "kernel": kernel,
-            "work": "the certificate's layer-evaluations x the FP64 element + Schur step's "
-                    "149.1 flops each",
+            "work": "the search's FP32 layer-evaluations x the FP32 element + Schur step's "
+                    "129.8 flops each",
             "peak_source": ("derived: 4 warp instructions issued/clk/SM x SMs x 2070 MHz / "
-                            f"{wi} warp instructions per layer-evaluation (ncu) x 149.1 flops"
+                            f"{wi} warp instructions per layer-evaluation (ncu) x 129.8 flops"
                             if peak_issue else
-                            "derived: 2 DFMA/clk/SM x 2 flop x SMs x 2070 MHz"),
+                            "derived: 128 FFMA/clk/SM x 2 flop x SMs x 2070 MHz"),
             "warp_instructions_per_layer_eval": wi,
-            "fp64_peak": peak64 / 1e12, "frac_of_fp64_peak": achieved / peak64,
-            "frac_of_fp64_microbenchmark": achieved / micro,
-            "layer_evals_per_launch": e64, "flops_per_layer_eval": F_LAYER_FLOPS,
-            "layer_evals_per_s": e64 / t0,
-            "fp64_flops_executed_per_layer_eval": F_LAYER_FLOPS_EXECUTED64,
-            "fp64_pipe_frac_executed": e64 * F_LAYER_FLOPS_EXECUTED64 / t0 / peak64,
+            "fp32_peak": peak32 / 1e12, "frac_of_fp32_peak": achieved / peak32,
+            "fp64_peak": peak64 / 1e12,
+            "layer_evals_per_launch": e32, "flops_per_layer_eval": F_LAYER_FLOPS_FP32,
+            "layer_evals_per_s": e32 / t0,
             "kernel_ms": t0 * 1e3,
-            "search_layer_evals_fp32": e32,
-            "search_fp32_frac_of_fp32_peak": e32 * F_LAYER_FLOPS_FP32 / t32 / peak32,
-            "search_frac_of_issue_ceiling": (
-                e32 / t32 / (ISSUE_PER_CLK_SM * sms * SM_MAX_MHZ * 1e6 /
-                             SEARCH_WARP_INSTR_PER_LAYER_EVAL[workload])
-                if split and workload in SEARCH_WARP_INSTR_PER_LAYER_EVAL else None),
+            "certificate_layer_evals": e64,
             "fallback_check_layer_evals_fp64": e64_fb,
             "linear_scan_layer_evals": linear,
             "linear_scan_over_counting_evals": linear / max(1, e32 + e64 + e64_fb),
