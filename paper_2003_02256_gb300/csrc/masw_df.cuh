@@ -847,7 +847,7 @@ __device__ __forceinline__ int det_inertia_t(const float* __restrict__ laydf,
     return cnt + last_pivot_inertia(lay + N * LAYER_STRIDE, c2, st);
 }
 
-// det_inertia_dd of four points by the four groups of 8 lanes of a warp, for
+// det_inertia_t of four points by the four groups of 8 lanes of a warp, for
 // short lists: a group's lanes take the elements of 8 layers side by side
 // (three quarters of a layer-evaluation) and pass them through shared memory
 // (`sh`: DD_GROUP_FLOATS floats of the group's own), then every lane runs the
@@ -857,15 +857,17 @@ __device__ __forceinline__ int det_inertia_t(const float* __restrict__ laydf,
 // group's count.
 constexpr int DD_GROUP = 8;
 constexpr int DD_GROUP_FLOATS = DD_GROUP * 14;
-static __device__ __noinline__ int det_inertia_dd_group(const float* __restrict__ laydf,
-                                                        const double* __restrict__ lay, int N,
-                                                        double k, double c, float* sh) {
+template <bool DD>
+__device__ __forceinline__ int det_inertia_group_t(const float* __restrict__ laydf,
+                                                   const double* __restrict__ lay, int N, double k,
+                                                   double c, float* sh) {
     const int gl = threadIdx.x & (DD_GROUP - 1);
     const double c2 = c * c;
     const DF kd = from_double(k), cd = from_double(c);
     const DF c2d = dmul(cd, cd);
     const DF ic2d = drcp(c2d);
     HStateDD sd{dfc(0.0f), dfc(0.0f), dfc(0.0f), dfc(1.0f)};
+    HState st{0.0, 0.0, 0.0, 1.0};
     int cnt = 0;
     bool good = true;
     const int most = __reduce_max_sync(0xffffffffu, N);
@@ -882,21 +884,36 @@ static __device__ __noinline__ int det_inertia_dd_group(const float* __restrict_
         for (int i = 0; i < steps; ++i) {
             if (j0 + i < N) {
                 const LayerNumDD nd = *reinterpret_cast<const LayerNumDD*>(sh + i * 14);
-                const bool f_neg = (sd.w.hi < 0.0f) != (nd.Dh.hi < 0.0f);  // sign of w Dh
-                DF s00;
                 bool ok;
-                const DF det = schur_layer_dd(sd, nd, &ok, &s00);
+                if (DD) {
+                    const bool f_neg = (sd.w.hi < 0.0f) != (nd.Dh.hi < 0.0f);  // sign of w Dh
+                    DF s00;
+                    const DF det = schur_layer_dd(sd, nd, &ok, &s00);
+                    cnt += det.hi < 0.0f
+                               ? 1
+                               : (det.hi > 0.0f ? (((s00.hi < 0.0f) != f_neg) ? 2 : 0) : 1);
+                } else {
+                    const LayerNum n{to_double(nd.Dh), to_double(nd.n00), to_double(nd.n01),
+                                     to_double(nd.n11), to_double(nd.ce), to_double(nd.cf),
+                                     to_double(nd.cg)};
+                    const bool f_neg = wprod_lt0(st.w, n.Dh);
+                    double sv[3];
+                    const double det = schur_layer(st, n, &ok, sv);
+                    cnt += lt0(det) ? 1 : (gt0(det) ? ((lt0(sv[0]) != f_neg) ? 2 : 0) : 1);
+                }
                 good = good && ok;
-                cnt += det.hi < 0.0f ? 1
-                                     : (det.hi > 0.0f ? (((s00.hi < 0.0f) != f_neg) ? 2 : 0) : 1);
             }
         }
         __syncwarp();
     }
-    if (N == 0 || !good) return -1;
-    return cnt + last_pivot_inertia(lay + N * LAYER_STRIDE, c2,
-                                    HState{to_double(sd.p00), to_double(sd.p01), to_double(sd.p11),
-                                           to_double(sd.w)});
+    if ((DD && N == 0) || !good) return -1;
+    if (DD) st = HState{to_double(sd.p00), to_double(sd.p01), to_double(sd.p11), to_double(sd.w)};
+    return cnt + last_pivot_inertia(lay + N * LAYER_STRIDE, c2, st);
+}
+static __device__ __noinline__ int det_inertia_dd_group(const float* __restrict__ laydf,
+                                                        const double* __restrict__ lay, int N,
+                                                        double k, double c, float* sh) {
+    return det_inertia_group_t<true>(laydf, lay, N, k, c, sh);
 }
 
 // Out of line: each is called from several places, and one copy of the
@@ -985,6 +1002,40 @@ static __device__ __noinline__ int mode_count_T_df(const float* __restrict__ lay
     for (int j = 0; j < N; ++j) j0 += clamped_modes(lay + j * LAYER_STRIDE, k, c2);
     *s_out = s;
     return s < 0 ? -1 : s + 2 * j0;
+}
+
+// mode_count_T_df by 8 lanes a point (det_inertia_group_t; the clamped modes a
+// layer per lane): same arithmetic, same counts. The FP64 pipe does every
+// lane's Schur step, so it is for lists short enough for one warp an item.
+static __device__ __noinline__ int mode_count_T_df_group(const float* __restrict__ laydf,
+                                                         const double* __restrict__ lay, int N,
+                                                         double k, double c, float* sh, int* s_out) {
+    const int s = det_inertia_group_t<false>(laydf, lay, N, k, c, sh);
+    const double c2 = c * c;
+    int j0 = 0;
+    for (int j = threadIdx.x & (DD_GROUP - 1); j < N; j += DD_GROUP)
+        j0 += clamped_modes(lay + j * LAYER_STRIDE, k, c2);
+    for (int d = DD_GROUP / 2; d; d >>= 1) j0 += __shfl_xor_sync(0xffffffffu, j0, d);
+    *s_out = s;
+    return s < 0 ? -1 : s + 2 * j0;
+}
+
+// The three-point check of a mode count by a warp: T and s at V[0] (p0),
+// V[n-1] (pa; V[nlim-1] for n < 1) and V[n] (pb, n >= 1), 8 lanes a point.
+// `sh`: four times DD_GROUP_FLOATS floats of the warp's own.
+__device__ __forceinline__ void check_points_group(const float* __restrict__ laydf,
+                                                   const double* __restrict__ lay, int N, double k,
+                                                   double c0, double dc, int n, int nlim, float* sh,
+                                                   int T[3], int s[3]) {
+    const int q = (threadIdx.x & 31) / DD_GROUP;
+    const int pt = q == 0 ? 0 : q == 1 ? (n >= 1 ? n - 1 : nlim - 1) : q == 2 && n >= 1 ? n : -1;
+    int sv;
+    const int Tv = mode_count_T_df_group(laydf, lay, pt >= 0 ? N : 0, k, grid_c(c0, dc, max(pt, 0)),
+                                         sh + q * DD_GROUP_FLOATS, &sv);
+    for (int i = 0; i < 3; ++i) {
+        T[i] = __shfl_sync(0xffffffffu, Tv, i * DD_GROUP);
+        s[i] = __shfl_sync(0xffffffffu, sv, i * DD_GROUP);
+    }
 }
 
 }  // namespace masw

@@ -417,17 +417,53 @@ __device__ __forceinline__ void after_previous() {
     cudaTriggerProgrammaticLaunchCompletion();
 }
 
+// The check of a short list, at most one item per warp of the grid, 8 lanes per
+// point: 750 items of up to 30 layers take a third of the four-lane form's
+// latency (701 ragged models 742-777 -> 682-729 us). Out of line, and the kernel's
+// parameters by reference from constant memory: inlined, the long lists' code
+// was slower (256 leaky models 4.25 -> 4.34 ms).
+static __device__ __noinline__ void verify_short_list(const DevBatch& b, const ScanOut& o,
+                                                      const int32_t* n32, const int32_t* list,
+                                                      int total, int32_t* search,
+                                                      int32_t* n_search) {
+    __shared__ __align__(8) float s_dd[4][4 * DD_GROUP_FLOATS];
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (t >= total) return;
+    const int item = list[t];
+    const int m = b.item_model[item];
+    const int lo = b.model_loff[m], nlim = b.model_nlim[m], n = n32[item];
+    if (nlim < 2) {
+        if ((threadIdx.x & 31) == 0) write_result(b, o, item, -1);
+        return;
+    }
+    int T[3], sv[3];
+    check_points_group(records_df(b, lo), b.layers + (size_t)lo * LAYER_STRIDE,
+                       b.model_loff[m + 1] - lo - 1, b.k[item], b.c0, b.dc, n, nlim,
+                       s_dd[threadIdx.x >> 5], T, sv);
+    if (threadIdx.x & 31) return;
+    if (route_level(b.route) < 2 && mode_count_verified(n, T[0], T[1], T[2]))
+        write_result(b, o, item, n >= 1 ? n : -1);
+    else
+        search[atomicAdd(n_search, 1)] = item;
+}
+
 // The same check over a device-counted list (the fallback items of the
 // counting search), four lanes per item so that its three FP64 evaluations
 // run side by side (a lone evaluation is a long dependent FP64 chain; a few
 // listed items are latency-bound), grid-stride over the list.
-__global__ void __launch_bounds__(128) verify64_list_kernel(DevBatch b, ScanOut o, const int32_t* n32,
+__global__ void __launch_bounds__(128) verify64_list_kernel(const __grid_constant__ DevBatch b,
+                                                            const __grid_constant__ ScanOut o,
+                                                            const int32_t* n32,
                                                             const int32_t* list,
                                                             const int32_t* n_list,
                                                             int32_t* search, int32_t* n_search) {
     after_previous();
     const int total = *n_list;
     const int lane = threadIdx.x & 31;
+    if (32 * total <= (int)(gridDim.x * blockDim.x)) {
+        verify_short_list(b, o, n32, list, total, search, n_search);
+        return;
+    }
     const int sub = lane & 3;
     const int q0 = lane & 28;
     const unsigned quad = 0xFu << q0;
@@ -1084,7 +1120,7 @@ static cudaError_t launch_tail(const DevBatch& b, const ScanOut& o, const ScanPl
                         (size_t)p.stage_layers * LAYER_STRIDE32 * sizeof(float), s, prio, false, b,
                         layers32, n32, fallback, counters + 3, counters + 4, p.stage_layers);
         if (e != cudaSuccess) return e;
-        e = launch_prio(verify64_list_kernel, std::max(1, std::min(p.blocks, (4 * n + 127) / 128)),
+        e = launch_prio(verify64_list_kernel, (int)std::max(1LL, std::min<long long>(p.blocks, (32LL * n + 127) / 128)),
                         128, 0, s, prio, early, b, o, n32, fallback, counters + 3, search,
                         counters + 5);
         if (e != cudaSuccess) return e;
