@@ -756,8 +756,8 @@ def measure(args, torch, masw, workload, n_models, rank, world, with_plain=True)
             "step_ms_median": float(np.median(step_ms)), "clocks": clk.summary(),
             "roofline": roofline, "plan": plan.as_dict(), "plain": plain, "e2e": e2e,
             "found_fraction": float(np.mean(st == 0)),
-            "launches_per_step": {0: 2, 1: 5,
-                                  2: (6, 8, 12)[plan.count_split]}[plan.precision]}
+            "launches_per_step": {0: 2, 1: 6,
+                                  2: (7, 9, 12)[plan.count_split]}[plan.precision]}
 
 
 def run_extras(args, masw, torch):
@@ -1225,8 +1225,9 @@ def main():
                 "clocks": r["clocks"],
                 "e2e": r["e2e"],
                 # per step: the scan's kernels (precision 0: scan; 1: screen, check,
-                # mode-count search, re-scan; 2: counting search + certificate,
-                # fallback scan, check, mode-count search, re-scan) and the misfit
+                # sign scan, mode-count search, re-scan; 2: counting search +
+                # certificate, fallback scan, check, sign scan, mode-count search,
+                # re-scan, the last three twice with the second stream) and the misfit
                 "gpu_launches": r["launches_per_step"] * args.steps,
                 "roofline": r["roofline"],
                 "cpu_baseline": cpu,
