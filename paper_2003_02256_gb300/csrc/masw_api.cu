@@ -1113,7 +1113,9 @@ static int run_roots(masw_batch* B) {
     int rc;
     if ((rc = ensure(&B->d_croot, B->n_items))) return rc;
     if ((rc = run_scan(B))) return rc;
-    CK(launch_refine(B->dev(false), B->d_layers32, B->d_idx, 1e-13, B->d_croot, B->stream));
+    // (the scan's search list is done with: it takes the flags)
+    CK(launch_refine(B->dev(false), B->d_layers32, B->d_idx, 1e-13, B->d_croot, B->d_search,
+                     B->stream));
     return MASW_OK;
 }
 
@@ -1123,7 +1125,8 @@ static int run_root_grad(masw_batch* B) {
         (rc = ensure(&B->d_bs, root_grad_scratch((int)B->n_items, B->max_layers, B->sm_count))))
         return rc;
     if ((rc = run_roots(B))) return rc;
-    CK(launch_root_grad(B->dev(false), B->d_croot, B->d_rows, B->d_bs, B->sm_count, B->stream));
+    CK(launch_root_grad(B->dev(false), B->d_croot, B->d_search, B->d_rows, B->d_bs, B->max_layers,
+                        B->sm_count, B->stream));
     return MASW_OK;
 }
 

@@ -140,11 +140,12 @@ cudaError_t launch_det_eval(const DevBatch& b, int n, const int32_t* item, const
 cudaError_t launch_mode_count(const DevBatch& b, int n, const int32_t* item, const double* c,
                               int32_t* s, int32_t* j0, cudaStream_t st);
 cudaError_t launch_refine(const DevBatch& b, const float* layers32, const int32_t* idx,
-                          double rel_tol, double* croot, cudaStream_t s);
-// scratch: root_grad_scratch doubles.
+                          double rel_tol, double* croot, int32_t* flag, cudaStream_t s);
+// flag: launch_refine's, per item; scratch: root_grad_scratch doubles.
 size_t root_grad_scratch(int n_items, int max_layers, int sms);
-cudaError_t launch_root_grad(const DevBatch& b, const double* croot, double* rows, double* scratch,
-                             int sms, cudaStream_t s);
+cudaError_t launch_root_grad(const DevBatch& b, const double* croot, const int32_t* flag,
+                             double* rows, double* scratch, int max_layers, int sms,
+                             cudaStream_t s);
 cudaError_t launch_misfit(const DevBatch& b, const double* ct, const double* ce, int kind,
                           double sigma, double* misfit, double* dphi_dc, cudaStream_t s);
 cudaError_t launch_grad_reduce(const DevBatch& b, const double* rows, const double* dphi_dc,

@@ -2019,11 +2019,12 @@ __device__ __forceinline__ double det_rel(const double* __restrict__ lay, int N,
 // A root's bracket narrowed on the FP32 count (inertia_bound_f's recurrence,
 // no bound): [a, bq] inside [lo, hi] with the count's parity changing across
 // it, a few FP32 steps wide, split in three per step by the pair's lanes. The
-// caller checks the FP64 determinant's signs at its ends. Returns false unless
+// caller checks the FP64 determinant's signs at its ends. Returns 1 when
 // the count rises by one from lo to hi with no clamped mode between them: a
 // sign change may also be a pole's, and with three roots, or roots and poles,
-// in one grid interval the one taken would depend on the path there.
-static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ lay32, int N,
+// in one grid interval the one taken would depend on the path there (-1). 0: no
+// rise seen, the root lies within FP32 rounding of an end.
+static __device__ __noinline__ int bracket_root_f32(const float* __restrict__ lay32, int N,
                                                      float kf, float lo, float hi, int half,
                                                      unsigned pair, float* a_out, float* b_out) {
     float a = lo, bq = hi;
@@ -2033,7 +2034,9 @@ static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ l
     for (int j = 0; j < N; ++j)
         j0 += clamped_modes_bound_f(lay32 + j * LAYER_STRIDE32, kf, c * c, &sure);
     const int oth = __shfl_xor_sync(pair, own, 1), j0_oth = __shfl_xor_sync(pair, j0, 1);
-    if ((half ? own - oth : oth - own) != 1 || j0 != j0_oth) return false;
+    const int rise = half ? own - oth : oth - own;
+    if (j0 != j0_oth || (rise & ~1)) return -1;
+    if (rise == 0) return 0;
     const int par_a = (half ? oth : own) & 1;
     // down to two FP32 steps of the velocity (2^-22 relative): the count's own
     // error is below that (about 1e-8 relative, from its misses next to roots)
@@ -2055,7 +2058,7 @@ static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ l
     }
     *a_out = a;
     *b_out = bq;
-    return true;
+    return 1;
 }
 
 // Refined root inside [V[idx-1], V[idx]] (the change located by the scan) to
@@ -2069,6 +2072,7 @@ static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ l
 // nearer point replaces the end of its sign, and an end kept twice in a row
 // has its value halved, so both ends converge. Every 8th step uses the
 // midpoint, so the bracket also shrinks at least as fast as in bisection.
+// flag: 1 for an item whose interval holds no simple root, for the adjoint.
 // Returns that secant point, or the midpoint of a bracket within the
 // tolerance; an exact zero returns its point.
 // Bound by the FP64 pipe: from the scan's bracket, closed by points a quarter
@@ -2077,7 +2081,7 @@ static __device__ __noinline__ bool bracket_root_f32(const float* __restrict__ l
 // wavelengths), from the FP32 bracket 2 (1.22 ms).
 __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __restrict__ layers32,
                                                      const int32_t* __restrict__ idx,
-                                                     double rel_tol, double* croot) {
+                                                     double rel_tol, double* croot, int32_t* flag) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int it = t >> 1;
     if (it >= b.n_items) return;  // both lanes of a pair leave together
@@ -2086,7 +2090,10 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __
     const int id = idx[it];
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     if (id < 1) {
-        if (!half) croot[it] = nan;
+        if (!half) {
+            croot[it] = nan;
+            flag[it] = 0;
+        }
         return;
     }
     const int m = b.item_model[it];
@@ -2096,11 +2103,13 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __
     const double k = b.k[it];
     const double v_lo = grid_c(b.c0, b.dc, id - 1), v_hi = grid_c(b.c0, b.dc, id);
     double lo = v_lo, hi = v_hi;
-    bool narrow = false;
+    bool narrow = false, simple = true;
     if (layers32) {
         float a, c;
-        narrow = bracket_root_f32(layers32 + (size_t)lo_rec * LAYER_STRIDE32, N, (float)k,
+        const int found = bracket_root_f32(layers32 + (size_t)lo_rec * LAYER_STRIDE32, N, (float)k,
                                   (float)v_lo, (float)v_hi, half, pair, &a, &c);
+        simple = found >= 0;
+        narrow = found > 0;
         if (narrow) {
             const double pad = 1.8e-7 * v_hi;
             lo = fmax(v_lo, (double)a - pad);
@@ -2184,13 +2193,17 @@ __global__ void __launch_bounds__(128) refine_kernel(DevBatch b, const float* __
         }
         if (!(result == result)) result = 0.5 * (lo + hi);
     }
-    if (!half) croot[it] = result;
+    if (!half) {
+        croot[it] = result;
+        flag[it] = simple ? 0 : 1;
+    }
 }
 
 cudaError_t launch_refine(const DevBatch& b, const float* layers32, const int32_t* idx,
-                          double rel_tol, double* croot, cudaStream_t s) {
+                          double rel_tol, double* croot, int32_t* flag, cudaStream_t s) {
     if (b.n_items <= 0) return cudaSuccess;
-    refine_kernel<<<(2 * b.n_items + 127) / 128, 128, 0, s>>>(b, layers32, idx, rel_tol, croot);
+    refine_kernel<<<(2 * b.n_items + 127) / 128, 128, 0, s>>>(b, layers32, idx, rel_tol, croot,
+                                                              flag);
     return cudaGetLastError();
 }
 
@@ -2221,6 +2234,7 @@ constexpr int ROOT_THREADS = 64;
 constexpr int ROOT_SLOTS = 13;
 __global__ void __launch_bounds__(ROOT_THREADS) root_grad_kernel(DevBatch b,
                                                                  const double* __restrict__ croot,
+                                                                 const int32_t* __restrict__ flag,
                                                                  double* rows, double* scratch) {
     const int tid = blockIdx.x * ROOT_THREADS + threadIdx.x;
     const int nt = gridDim.x * ROOT_THREADS;
@@ -2229,6 +2243,7 @@ __global__ void __launch_bounds__(ROOT_THREADS) root_grad_kernel(DevBatch b,
         return scratch[((size_t)node * ROOT_SLOTS + slot) * nt + tid];
     };
     for (int it = tid; it < b.n_items; it += nt) {
+        if (flag[it]) continue;  // root_grad_duals_kernel
         const int m = b.item_model[it];
         const int lo_rec = b.model_loff[m];
         const int N = b.model_loff[m + 1] - lo_rec - 1;
@@ -2352,6 +2367,171 @@ __global__ void __launch_bounds__(ROOT_THREADS) root_grad_kernel(DevBatch b,
     }
 }
 
+// Items whose interval holds no simple root (refine_kernel's flag: a pole, three
+// roots): the adjoint is then a quotient of two singular terms, and which
+// rounding it takes shows in its digits, so these few keep the plain form:
+// general 2x2 blocks and the element in dual numbers. `ws`: 24 doubles per node.
+struct M2 { double a, b, c, d; };
+__device__ __forceinline__ M2 mmul(M2 x, M2 y) {
+    return {x.a * y.a + x.b * y.c, x.a * y.b + x.b * y.d, x.c * y.a + x.d * y.c, x.c * y.b + x.d * y.d};
+}
+__device__ __forceinline__ M2 madd(M2 x, M2 y) { return {x.a + y.a, x.b + y.b, x.c + y.c, x.d + y.d}; }
+__device__ __forceinline__ M2 msub(M2 x, M2 y) { return {x.a - y.a, x.b - y.b, x.c - y.c, x.d - y.d}; }
+__device__ __forceinline__ double mdet(M2 x) { return x.a * x.d - x.b * x.c; }
+// x^-1 y
+__device__ __forceinline__ M2 msolve(M2 x, M2 y) {
+    double id = 1.0 / mdet(x);
+    M2 adj = {x.d * id, -x.b * id, -x.c * id, x.a * id};
+    return mmul(adj, y);
+}
+__device__ __forceinline__ void mvsolve(M2 x, double v0, double v1, double* o0, double* o1) {
+    double id = 1.0 / mdet(x);
+    *o0 = (x.d * v0 - x.b * v1) * id;
+    *o1 = (-x.c * v0 + x.a * v1) * id;
+}
+__device__ __forceinline__ void ld(const double* p, M2* m) { *m = {p[0], p[1], p[2], p[3]}; }
+__device__ __forceinline__ void st(double* p, M2 m) { p[0] = m.a; p[1] = m.b; p[2] = m.c; p[3] = m.d; }
+
+// Element blocks of layer j at (k, c), k dropped: K11, K12 (K22 and K21 follow
+// from the layer's symmetry: K22 = [[A, -B], [-B, Dd]], K21 = K12^T).
+__device__ __forceinline__ void elem_blocks(const double* L, double k, double c2, M2* K11, M2* K12,
+                                            M2* K21, M2* K22) {
+    LayerNum n = layer_numerators(L, k, c2, inv_c2(c2));
+    double id = 1.0 / n.Dh;
+    double A = n.n00 * id, B = n.n01 * id, Dd = n.n11 * id;
+    double E = n.ce * id, F = n.cf * id, G = n.cg * id;
+    *K11 = {A, B, B, Dd};
+    *K22 = {A, -B, -B, Dd};
+    *K12 = {E, F, -F, G};
+    *K21 = {E, -F, F, G};
+}
+
+// The blocks of elem_blocks from its six stored entries (A, B, Dd, E, F, G).
+__device__ __forceinline__ void stored_blocks(const double* E6, M2* K11, M2* K12, M2* K21, M2* K22) {
+    const double A = E6[0], B = E6[1], Dd = E6[2], E = E6[3], F = E6[4], G = E6[5];
+    *K11 = {A, B, B, Dd};
+    *K22 = {A, -B, -B, Dd};
+    *K12 = {E, F, -F, G};
+    *K21 = {E, -F, F, G};
+}
+
+static __device__ __noinline__ void root_grad_duals(const DevBatch& b, const double* croot, double* rows,
+                                                    double* ws, int it) {
+    int m = b.item_model[it];
+    int lo_rec = b.model_loff[m];
+    int N = b.model_loff[m + 1] - lo_rec - 1;
+    double* row = rows + b.grad_off[it];
+    const double nan = __longlong_as_double(0x7ff8000000000000LL);
+    double c = croot[it];
+    if (!(c == c)) {
+        for (int p = 0; p < 2 * N + 1; ++p) row[p] = nan;
+        return;
+    }
+    const double* lay = b.layers + (size_t)lo_rec * LAYER_STRIDE;
+    double k = b.k[it];
+    double c2 = c * c;
+    // node j slot: [0..3] S_j (top-down), [4..7] M_j = B_{j+1} + K22_j,
+    //              [8..11] B_j (bottom-up), [12..15] P_j,
+    //              [16..21] layer j's element entries (A, B, Dd, E, F, G)
+    M2 P = {0.0, 0.0, 0.0, 0.0};
+    for (int j = 0; j < N; ++j) {
+        M2 K11, K12, K21, K22;
+        elem_blocks(lay + j * LAYER_STRIDE, k, c2, &K11, &K12, &K21, &K22);
+        double* E6 = ws + 24 * j + 16;
+        E6[0] = K11.a; E6[1] = K11.b; E6[2] = K11.d; E6[3] = K12.a; E6[4] = K12.b; E6[5] = K12.d;
+        M2 S = madd(P, K11);
+        st(ws + 24 * j, S);
+        st(ws + 24 * j + 12, P);
+        P = msub(K22, mmul(K21, msolve(S, K12)));
+    }
+    st(ws + 24 * N + 12, P);
+    HalfNum hn = halfspace_numerators(lay + N * LAYER_STRIDE, c2);
+    double iden = 1.0 / hn.den;
+    M2 Bv = {hn.m00 * iden, hn.m01 * iden, hn.m01 * iden, hn.m11 * iden};
+    st(ws + 24 * N + 8, Bv);
+    for (int j = N - 1; j >= 0; --j) {
+        M2 K11, K12, K21, K22;
+        stored_blocks(ws + 24 * j + 16, &K11, &K12, &K21, &K22);
+        M2 Mj = madd(Bv, K22);
+        st(ws + 24 * j + 4, Mj);
+        Bv = msub(K11, mmul(K12, msolve(Mj, K21)));
+        st(ws + 24 * j + 8, Bv);
+    }
+    // twist node: most singular condensed block
+    int js = N;
+    double best = 1e300;
+    for (int j = 0; j <= N; ++j) {
+        M2 Pj, Bj;
+        ld(ws + 24 * j + 12, &Pj);
+        ld(ws + 24 * j + 8, &Bj);
+        M2 G = madd(Pj, Bj);
+        double nrm = G.a * G.a + G.b * G.b + G.c * G.c + G.d * G.d;
+        double sng = fabs(mdet(G)) / nrm;
+        if (sng < best) { best = sng; js = j; }
+    }
+    M2 G;
+    {
+        M2 Pj, Bj;
+        ld(ws + 24 * js + 12, &Pj);
+        ld(ws + 24 * js + 8, &Bj);
+        G = madd(Pj, Bj);
+    }
+    // null vector of the 2x2 G from its larger row
+    double nx, nz;
+    if (G.a * G.a + G.b * G.b >= G.c * G.c + G.d * G.d) { nx = -G.b; nz = G.a; }
+    else { nx = -G.d; nz = G.c; }
+    double nn = fmax(fabs(nx), fabs(nz));
+    nx /= nn; nz /= nn;
+    // store u_j in the P slot (no longer needed): [12], [13]
+    ws[24 * js + 12] = nx;
+    ws[24 * js + 13] = nz;
+    for (int j = js - 1; j >= 0; --j) {  // upward: u_j = -S_j^-1 K12_j u_{j+1}
+        M2 K11, K12, K21, K22, S;
+        stored_blocks(ws + 24 * j + 16, &K11, &K12, &K21, &K22);
+        ld(ws + 24 * j, &S);
+        double x = ws[24 * (j + 1) + 12], z = ws[24 * (j + 1) + 13];
+        double v0 = K12.a * x + K12.b * z, v1 = K12.c * x + K12.d * z, o0, o1;
+        mvsolve(S, v0, v1, &o0, &o1);
+        ws[24 * j + 12] = -o0;
+        ws[24 * j + 13] = -o1;
+    }
+    for (int j = js + 1; j <= N; ++j) {  // downward: u_j = -M_{j-1}^-1 K21_{j-1} u_{j-1}
+        M2 K11, K12, K21, K22, Mj;
+        stored_blocks(ws + 24 * (j - 1) + 16, &K11, &K12, &K21, &K22);
+        ld(ws + 24 * (j - 1) + 4, &Mj);
+        double x = ws[24 * (j - 1) + 12], z = ws[24 * (j - 1) + 13];
+        double v0 = K21.a * x + K21.b * z, v1 = K21.c * x + K21.d * z, o0, o1;
+        mvsolve(Mj, v0, v1, &o0, &o1);
+        ws[24 * j + 12] = -o0;
+        ws[24 * j + 13] = -o1;
+    }
+    // implicit-function rule with dual-number element derivatives
+    HalfD H = halfspace_d(lay + N * LAYER_STRIDE, c);
+    D4 qh = half_quad(H, ws[24 * N + 12], ws[24 * N + 13]);
+    double den = qh.d0;
+    row[N] = qh.d1;
+    for (int j = 0; j < N; ++j) {
+        ElemD K = layer_element_d(lay + j * LAYER_STRIDE, k, c);
+        D4 q = elem_quad(K, ws[24 * j + 12], ws[24 * j + 13], ws[24 * (j + 1) + 12],
+                         ws[24 * (j + 1) + 13]);
+        den += q.d0;
+        row[j] = q.d1;
+        row[N + 1 + j] = q.d2;
+    }
+    double inv = -1.0 / den;
+    for (int p = 0; p < 2 * N + 1; ++p) row[p] *= inv;
+}
+
+__global__ void __launch_bounds__(64) root_grad_duals_kernel(const __grid_constant__ DevBatch b,
+                                                             const double* croot, const int32_t* flag,
+                                                             double* rows, double* scratch,
+                                                             int threads, int stride) {
+    const int tid = blockIdx.x * 64 + threadIdx.x;
+    if (tid >= threads) return;
+    for (int it = tid; it < b.n_items; it += threads)
+        if (flag[it]) root_grad_duals(b, croot, rows, scratch + (size_t)tid * stride, it);
+}
+
 // Threads of root_grad_kernel for n_items items: at most 256 per SM (the FP64
 // pipe is busy with fewer), so that the scratch of models of up to 23 layers
 // stays within the 129 MB L2.
@@ -2363,11 +2543,20 @@ size_t root_grad_scratch(int n_items, int max_layers, int sms) {
     return (size_t)root_grad_threads(n_items, sms) * ROOT_SLOTS * std::max(max_layers, 1);
 }
 
-cudaError_t launch_root_grad(const DevBatch& b, const double* croot, double* rows, double* scratch,
-                             int sms, cudaStream_t s) {
+cudaError_t launch_root_grad(const DevBatch& b, const double* croot, const int32_t* flag,
+                             double* rows, double* scratch, int max_layers, int sms,
+                             cudaStream_t s) {
     if (b.n_items <= 0) return cudaSuccess;
     root_grad_kernel<<<root_grad_threads(b.n_items, sms) / ROOT_THREADS, ROOT_THREADS, 0, s>>>(
-        b, croot, rows, scratch);
+        b, croot, flag, rows, scratch);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    // the same scratch, as many threads as it holds
+    const int stride = 24 * (max_layers + 1);
+    const int threads = (int)std::min<size_t>(
+        b.n_items, root_grad_scratch(b.n_items, max_layers, sms) / stride);
+    root_grad_duals_kernel<<<(threads + 63) / 64, 64, 0, s>>>(b, croot, flag, rows, scratch, threads,
+                                                              stride);
     return cudaGetLastError();
 }
 
